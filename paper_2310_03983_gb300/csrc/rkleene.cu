@@ -10,6 +10,7 @@
 // no CTA reads a tile another CTA is writing; the closed factor has a zero diagonal, so the
 // plain product already includes the old entry and needs no extra min.
 #include "closure.cuh"
+#include "gemm64.cuh"
 
 namespace apsp {
 
@@ -55,7 +56,9 @@ int gemm_aligned(void *C, int64_t ldc, const void *A, int64_t lda, const void *B
   p.no_trace = run_if != nullptr;
   const bool packed = !run_if && dtype == APSP_I32 && pk.scratch && K > 0 && pk.bytes >= packed_bytes(M, N, K) &&
                       (double)M * (double)N * (double)K >= kPacked16MinPairs;
-  if (!packed) return launch_tgemm(kModeGemm, acc, dtype, mA, mB, mC, p, s);
+  const bool small = gemm64_pays(M, N, K);
+  if (!packed)
+    return small ? launch_gemm64(acc, dtype, A, lda, B, ldb, p, s) : launch_tgemm(kModeGemm, acc, dtype, mA, mB, mC, p, s);
   // words[0], words[1]: largest finite entries of A and B; words[4]: set by the pack kernels
   // when their sum is below kCap16 (then every finite sum is exact in 16 bits).
   int *w = pk.words;
@@ -77,10 +80,12 @@ int gemm_aligned(void *C, int64_t ldc, const void *A, int64_t lda, const void *B
   q.arith16 = 1;
   q.run_if = w + 4;
   q.no_trace = 1;
-  if ((r = launch_tgemm(kModeGemm, acc, dtype, pA, pB, mC, q, s))) return r;
+  r = small ? launch_gemm64(acc, dtype, A16, lda16, B16, ldb16, q, s) : launch_tgemm(kModeGemm, acc, dtype, pA, pB, mC, q, s);
+  if (r) return r;
   p.skip = w + 4;
   p.no_trace = 1;
-  if ((r = launch_tgemm(kModeGemm, acc, dtype, mA, mB, mC, p, s))) return r;
+  r = small ? launch_gemm64(acc, dtype, A, lda, B, ldb, p, s) : launch_tgemm(kModeGemm, acc, dtype, mA, mB, mC, p, s);
+  if (r) return r;
   if (tev) trace_end(s, tev, kModeGemm, (double)M * (double)N * (double)K);
   return APSP_OK;
 }

@@ -9,7 +9,10 @@
 // commit read that word on the device and return at once when it is still set, so the whole
 // loop is enqueued up front without a host round trip per iteration (and can be captured in
 // a CUDA graph), yet stops doing work at convergence.
+#include <algorithm>
+
 #include "closure.cuh"
+#include "gemm64.cuh"
 
 namespace apsp {
 
@@ -46,12 +49,18 @@ int iters_for(int64_t n) {
 
 }  // namespace apsp
 
-extern "C" size_t apsp_squaring_workspace_bytes(int64_t n, int64_t ld, int dtype) {
-  using namespace apsp;
-  (void)dtype;
-  if (n <= 0) return 0;
+namespace apsp {
+// What a call cannot do without; the packed operands of small int32 matrices (last) are optional.
+static size_t squaring_required_bytes(int64_t n, int64_t ld) {
   const size_t mat = (size_t)round_up(n * round_up(n, 4) * 4, 256);
   return kFlagBytes + mat + (ld % 4 != 0 ? mat : 0);
+}
+}  // namespace apsp
+
+extern "C" size_t apsp_squaring_workspace_bytes(int64_t n, int64_t ld, int dtype) {
+  using namespace apsp;
+  if (n <= 0) return 0;
+  return squaring_required_bytes(n, ld) + (n <= kSquaring64MaxN ? squaring64_bytes(n, dtype) : 0);
 }
 
 extern "C" int apsp_squaring(void *d, int64_t n, int64_t ld, int dtype, const void *inf, int max_iters, void *ws,
@@ -66,7 +75,8 @@ extern "C" int apsp_squaring(void *d, int64_t n, int64_t ld, int dtype, const vo
   const int iters = max_iters == 0 ? iters_for(n) : max_iters;
   if (iters > kMaxIters) return APSP_ERR_ARG;
   const size_t need = apsp_squaring_workspace_bytes(n, ld, dtype);
-  if (ws && (ws_bytes < need || reinterpret_cast<uintptr_t>(ws) % 256 != 0)) return APSP_ERR_ARG;
+  const size_t base = squaring_required_bytes(n, ld);
+  if (ws && (ws_bytes < base || reinterpret_cast<uintptr_t>(ws) % 256 != 0)) return APSP_ERR_ARG;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   void *own = nullptr;
   if (!ws) {
@@ -74,7 +84,10 @@ extern "C" int apsp_squaring(void *d, int64_t n, int64_t ld, int dtype, const vo
       return APSP_ERR_NOMEM;
     }
     ws = own;
+    ws_bytes = need;
   }
+  void *packed = need > base && ws_bytes >= need ? reinterpret_cast<uint8_t *>(ws) + base : nullptr;
+  const bool small = n <= kSquaring64MaxN;
   int r = APSP_OK;
   uint8_t *wsp = reinterpret_cast<uint8_t *>(ws);
   int *words = reinterpret_cast<int *>(wsp);  // [0]: largest finite weight, [1]: 0, [8 + t]: unchanged flags
@@ -82,8 +95,8 @@ extern "C" int apsp_squaring(void *d, int64_t n, int64_t ld, int dtype, const vo
   const int64_t lde = round_up(n, 4);
   int *C = reinterpret_cast<int *>(wsp);
   wsp += round_up(n * lde * 4, 256);
-  if (cudaMemsetAsync(words, 0, 16, s) != cudaSuccess) r = APSP_ERR_CUDA;
-  if (!r && cudaMemsetAsync(words + kWordsUnchanged, 1, 4 * kMaxIters, s) != cudaSuccess) r = APSP_ERR_CUDA;
+  if (cudaMemsetAsync(words, 0, small ? kFlagBytes : 16, s) != cudaSuccess) r = APSP_ERR_CUDA;
+  if (!r && !small && cudaMemsetAsync(words + kWordsUnchanged, 1, 4 * kMaxIters, s) != cudaSuccess) r = APSP_ERR_CUDA;
   void *work = d;
   int64_t ldw = ld;
   if (!r && ld % 4 != 0) {  // the engine needs 16-byte rows: work on an aligned copy
@@ -91,12 +104,19 @@ extern "C" int apsp_squaring(void *d, int64_t n, int64_t ld, int dtype, const vo
     work = wsp;
     r = launch_copy2d(work, ldw, d, ld, n, n, s);
   }
-  if (!r) r = launch_normalise(work, n, ldw, dtype, inf_i, inf_f, dtype == APSP_I32 ? words : nullptr, s);
+  // Small matrices: the whole loop in one launch on 64 x 64 tiles (gemm64.cu), no more products than
+  // can change anything.
+  const int needed = std::min(iters, iters_for(n));
+  if (!r && small && needed > 0) {
+    r = squaring64(work, n, ldw, dtype, inf_i, inf_f, needed, words, C, lde, packed, s);
+  } else if (!r) {
+    r = launch_normalise(work, n, ldw, dtype, inf_i, inf_f, dtype == APSP_I32 ? words : nullptr, s);
+  }
   CUtensorMap mA, mB, mC;
   if (!r) r = make_operand_maps(work, n, n, ldw, dtype, &mA, &mB, nullptr);
   if (!r) r = make_operand_maps(C, n, n, lde, dtype, nullptr, nullptr, &mC);
   const int64_t cap = (int64_t)sm_count() * 8;
-  for (int t = 0; t < iters && !r; ++t) {
+  for (int t = 0; t < iters && !r && !small; ++t) {
     const int *skip = t > 0 ? words + kWordsUnchanged + t - 1 : nullptr;
     TileProblem p = {};
     p.M = n; p.N = n; p.K = n;

@@ -26,6 +26,7 @@
 #include <utility>
 
 #include "diag.cuh"
+#include "gemm64.cuh"
 #include "slab.cuh"
 #include "tgemm.cuh"
 
@@ -906,6 +907,7 @@ extern "C" int tropical_gemm(void *C, const void *A, const void *B, int64_t M, i
   // int32 with room for the packed copies: when the largest finite entries of A and B sum
   // below 0x3FFF (checked by the pack kernels on the device), the product runs on 16-bit pairs,
   // two (min,+) pairs per DPX operation; the plain launch then returns at once.
+  const bool small = gemm64_pays(M, N, K);
   void *tev = nullptr;
   const bool group = !r && dtype == APSP_I32 && K > 0 && ws_bytes >= kFlagBytes + p16;
   if (group && trace_on()) trace_begin(s, &tev);
@@ -924,12 +926,14 @@ extern "C" int tropical_gemm(void *C, const void *A, const void *B, int64_t M, i
       q.arith16 = 1;
       q.run_if = words + 4;
       q.no_trace = 1;
-      r = launch_tgemm(kModeGemm, accumulate != 0, dtype, pA, pB, mC, q, s);
+      r = small ? launch_gemm64(accumulate != 0, dtype, A16, lda16, B16, ldb16, q, s)
+                : launch_tgemm(kModeGemm, accumulate != 0, dtype, pA, pB, mC, q, s);
     }
     p.skip = words + 4;
     p.no_trace = 1;
   }
-  if (!r) r = launch_tgemm(kModeGemm, accumulate != 0, dtype, mA, mB, mC, p, s);
+  if (!r) r = small ? launch_gemm64(accumulate != 0, dtype, A, lda, B, ldb, p, s)
+                    : launch_tgemm(kModeGemm, accumulate != 0, dtype, mA, mB, mC, p, s);
   if (tev) trace_end(s, tev, kModeGemm, (double)M * (double)N * (double)K);
   ws_free(own, s);
   return r;
