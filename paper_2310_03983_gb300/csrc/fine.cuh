@@ -1,0 +1,25 @@
+// fine.cuh -- blocked Floyd-Warshall over 64 x 64 tiles for matrices too small to fill the GPU with
+// 128 x 128 tiles (fine.cu).
+#pragma once
+
+#include "tgemm.cuh"
+
+namespace apsp {
+
+// fw_loop closes matrices of kFineMinN < n <= kFineMaxN with 64-vertex blocks.  Up to 128 vertices the
+// 128-vertex loop is one launch over one tile; above kFineMaxN its larger tiles do more per load
+// (n = 3200: 2311 us against 2461 with 128-vertex blocks for int32, 2513 against 2544 with weights up
+// to 10^6, 2312 against 2648 for float32; n = 3300: 2623 against 2588, 2819 against 2662, 2626 against 2783).
+constexpr int64_t kFineMinN = 128, kFineMaxN = 3200;
+
+// Device words of the counters block (Bound::counters): all zero between launches.
+constexpr int kFineWords = 2 + 2 * 4;
+
+// Closes the n x n block at d (16-byte aligned, ld % 4 == 0, normalised) in place with
+// 1 + (number of 128-vertex blocks) launches after the first (one launch when n <= 128), the
+// launch structure of the 128-vertex loop.  wmax / wmult: the bound of the exact fp32 sequence for int32 storage (null: float32).
+// run_if (may be null): every launch returns at once unless *run_if is set.
+int fine_closure(void *d, int64_t n, int64_t ld, int dtype, int inf_i, const int *wmax, int64_t wmult,
+                 const int *run_if, int *counters, int trace_class, cudaStream_t s);
+
+}  // namespace apsp
