@@ -39,7 +39,7 @@ constexpr int kBThreads = 256;
 constexpr int kBStages = 4;
 constexpr int kBSlabInts = kSlabM * kSlabK;  // 4096 ints per A or B slab
 constexpr int kBTileInts = kSlabM * kSlabN;  // 16384 ints per 128 x 128 tile
-constexpr int kBSmemBytes = (2 * kBStages * kBSlabInts + kBTileInts + 512) * 4 + 256;
+constexpr int kBSmemBytes = (2 * kBStages * kBSlabInts + kBTileInts + kPairBufInts) * 4 + 256;
 
 struct BatchArgs {
   int *pool;
@@ -113,16 +113,17 @@ __device__ int normalise_graph(int *D, int n, int ld, const BatchArgs &a, int *r
 }
 
 // Phase 1: Eq. 1 on the bk x bk diagonal tile at (kb0, kb0), closed in registers (diag.cuh);
-// int32 graphs relax in int32 (exact), float32 graphs in fp32.
+// in fp32 for float32 graphs and int32 ones within the exact bound (f32), else in int32.
 template <typename S>
-__device__ void close_diag(int *D, int n, int ld, int kb0, int *buf) {
+__device__ void close_diag(int *D, int n, int ld, int kb0, bool f32, int *buf) {
   const int bk = min(kSlabM, n - kb0);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tm = (warp & 3) * 4 + (lane >> 3), tn = (warp >> 2) * 8 + (lane & 7);
   int *T = D + (int64_t)kb0 * ld + kb0;
   int r[8][8];
   load_tile_regs(r, T, ld, bk, tm, tn);
-  close_tile_regs<Store<S>::is_float>(r, bk, tm, tn, buf);
+  if (Store<S>::is_float || f32) close_tile_pairs<true>(r, bk, tm, tn, buf);
+  else close_tile_pairs<false>(r, bk, tm, tn, buf);
   store_tile_regs(r, T, ld, bk, tm, tn);
   __syncthreads();
 }
@@ -287,7 +288,7 @@ __device__ void close_blocked(int *D, int n, int ld, bool f32, int init_bits, in
                               int rank, int csize) {
   const int nb = (n + kSlabM - 1) / kSlabM;
   for (int kb = 0; kb < nb; ++kb) {
-    if (rank == 0) close_diag<S>(D, n, ld, kb * kSlabM, sT);
+    if (rank == 0) close_diag<S>(D, n, ld, kb * kSlabM, f32, sT);
     if (nb == 1) break;
     group_sync(csize);
     phase_tiles<false>(D, n, ld, kb, nb, 2 * (nb - 1), rank, csize, sA, sB, sC, f32, init_bits);

@@ -15,17 +15,20 @@
 #include "closure.cuh"
 #include "diag.cuh"
 #include "fine.cuh"
+#include "slab.cuh"
 
 namespace apsp {
 
 // Phase 1: Eq. 1 on the bk x bk diagonal tile, closed in registers by one 256-thread CTA
-// (diag.cuh).  int32 tiles are relaxed in int32 (exact for any weights), float32 in fp32.
+// (diag.cuh): float32 tiles in fp32, int32 ones in fp32 on their bit patterns within the exact bound
+// (wmax, mult as TileProblem's), else in int32.
 template <bool FLOAT>
-__global__ void __launch_bounds__(256) fw_diag_kernel(int *d, int64_t ld, int64_t n, int64_t kb, const int *run_if) {
+__global__ void __launch_bounds__(256) fw_diag_kernel(int *d, int64_t ld, int64_t n, int64_t kb, const int *wmax,
+                                                      int64_t mult, const int *run_if) {
   pdl_wait();
   pdl_trigger();
   if (run_if && !*run_if) return;
-  __shared__ __align__(16) int buf[512];
+  __shared__ __align__(16) int buf[kPairBufInts];
   const int64_t kb0 = kb * kBM;
   const int bk = (int)std::min<int64_t>(kBM, n - kb0);
   int *T = d + kb0 * ld + kb0;
@@ -33,15 +36,17 @@ __global__ void __launch_bounds__(256) fw_diag_kernel(int *d, int64_t ld, int64_
   const int tm = (warp & 3) * 4 + (lane >> 3), tn = (warp >> 2) * 8 + (lane & 7);
   int r[8][8];
   load_tile_regs(r, T, ld, bk, tm, tn);
-  close_tile_regs<FLOAT>(r, bk, tm, tn, buf);
+  if (FLOAT || (wmax && small_int_bound(wmax[0], mult, wmax[1]))) close_tile_pairs<true>(r, bk, tm, tn, buf);
+  else close_tile_pairs<false>(r, bk, tm, tn, buf);
   store_tile_regs(r, T, ld, bk, tm, tn);
 }
 
-int launch_fw_diag(void *d, int64_t ld, int64_t n, int64_t kb, int dtype, cudaStream_t s, const int *run_if) {
+static int launch_fw_diag(void *d, int64_t ld, int64_t n, int64_t kb, int dtype, const int *wmax, int64_t mult,
+                          cudaStream_t s, const int *run_if) {
   if (dtype == APSP_I32)
-    launch_pdl(fw_diag_kernel<false>, 1, 256, 0, s, reinterpret_cast<int *>(d), ld, n, kb, run_if);
+    launch_pdl(fw_diag_kernel<false>, 1, 256, 0, s, reinterpret_cast<int *>(d), ld, n, kb, wmax, mult, run_if);
   else
-    launch_pdl(fw_diag_kernel<true>, 1, 256, 0, s, reinterpret_cast<int *>(d), ld, n, kb, run_if);
+    launch_pdl(fw_diag_kernel<true>, 1, 256, 0, s, reinterpret_cast<int *>(d), ld, n, kb, wmax, mult, run_if);
   APSP_LAUNCH_CHECK();
   return APSP_OK;
 }
@@ -214,7 +219,7 @@ static int fw_loop(void *d, int64_t n, int64_t ld, int dtype, const CUtensorMap 
   p.run_if = run_if;
   p.trace_class = trace_class;
   for (int64_t kb = 0; kb < nb; ++kb) {
-    if ((kb == 0 || !counters) && (r = launch_fw_diag(d, ld, n, kb, dtype, s, run_if))) return r;
+    if ((kb == 0 || !counters) && (r = launch_fw_diag(d, ld, n, kb, dtype, p.wmax, p.wmult, s, run_if))) return r;
     if (nb == 1) break;
     p.kb = kb;
     if (kb == 0 || !counters) {
@@ -342,7 +347,7 @@ static int fw_wide_pass(void *d, int64_t n, int64_t ld, int dtype, int inf_i, Bo
     int *sub = D + kb0 * ld + kb0, *rowp = D + kb0 * ld, *colp = D + kb0;
     if (bt == 1) {  // phases 1 and 2 of a single-tile block, in place (as in the plain loop); with
                     // counters, those of every block after the first ran in the previous phase 3
-      if ((kbb == 0 || !b.counters) && (r = launch_fw_diag(d, ld, n, kbb, dtype, s, nullptr))) return r;
+      if ((kbb == 0 || !b.counters) && (r = launch_fw_diag(d, ld, n, kbb, dtype, p.wmax, p.wmult, s, nullptr))) return r;
       if (kbb == 0 || !b.counters) {
         TileProblem pp = p;
         pp.kb = kbb;

@@ -301,7 +301,7 @@ __global__ void __launch_bounds__(256, 2) group_diag_kernel(int *S, int64_t ldS,
   int nb = 0;
   graph_rows(gs, q, base, nb);
   if (nb <= kb) return;
-  __shared__ __align__(16) int buf[512];
+  __shared__ __align__(16) int buf[kPairBufInts];
   int *T = S + (base + (int64_t)kb * kBM) * ldS + (int64_t)kb * kBM;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tm = (warp & 3) * 4 + (lane >> 3), tn = (warp >> 2) * 8 + (lane & 7);
@@ -324,9 +324,9 @@ __global__ void __launch_bounds__(256, 2) group_diag_kernel(int *S, int64_t ldS,
         r[i][2 * j + 1] = (int)((unsigned)w[i][j] >> 16);
       }
   } else if (is_float) {
-    close_tile_regs<true>(r, bk, tm, tn, buf);
+    close_tile_pairs<true>(r, bk, tm, tn, buf);
   } else {
-    close_tile_regs<false>(r, bk, tm, tn, buf);
+    close_tile_pairs<false>(r, bk, tm, tn, buf);
   }
   store_tile_regs(r, T, ldS, kBM, tm, tn);
   if (pa) {  // the closed tile's part of this step's packed column and row panels

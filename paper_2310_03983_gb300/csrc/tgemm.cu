@@ -392,10 +392,10 @@ __device__ __forceinline__ void consume(const TileProblem &p, const Smem &sm, in
       for (int i = 0; i < 8; ++i)
 #pragma unroll
         for (int j = 0; j < 8; ++j) d[i][j] = AR::to(acc[i][j]);
-      if (fstore)
-        close_tile_regs<true, 1>(d, tc.m_valid, tm, tn, sm.dbuf);
+      if (fstore || (p.wmax && small_int_bound(p.wmax[0], p.wmult, p.wmax[1])))
+        close_tile_pairs<true, 1>(d, tc.m_valid, tm, tn, sm.dbuf);
       else
-        close_tile_regs<false, 1>(d, tc.m_valid, tm, tn, sm.dbuf);
+        close_tile_pairs<false, 1>(d, tc.m_valid, tm, tn, sm.dbuf);
 #pragma unroll
       for (int i = 0; i < 8; ++i)
 #pragma unroll

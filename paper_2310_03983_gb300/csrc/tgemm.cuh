@@ -19,8 +19,8 @@ constexpr int kAStageBytes = kBM * kBK * 4;         // A tile [128 m][32 k]
 constexpr int kBStageBytes = kBK * kBN * 4;         // B tile [32 k][128 n]
 constexpr int kCBytes = kBM * kBN * 4;              // C tile [128 m][128 n]
 // Shared memory: the stage ring, the C tile, 256 bytes of mbarriers and the tile-index ring, and
-// 2 KB of row / column buffers for the in-kernel diagonal closure (close_next).
-constexpr int kDiagBufBytes = 512 * 4;
+// 4 KB of row / column buffers for the in-kernel diagonal closure (close_next).
+constexpr int kDiagBufBytes = 1024 * 4;
 constexpr int kSmemBytes = kStages * (kAStageBytes + kBStageBytes) + kCBytes + 256 + kDiagBufBytes;
 
 // Which tiles a launch visits and where their operands live.
