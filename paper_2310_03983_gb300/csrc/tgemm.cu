@@ -838,6 +838,46 @@ static size_t packed16_bytes(int64_t M, int64_t N, int64_t K) {
 }
 }  // namespace apsp
 
+namespace apsp {
+// Smallest unaligned product that runs on aligned copies (3001 x 2503 x 1999 float32: 913 us against
+// 1619 with the plain-load kernel).  Below, the plain-load kernel's single launch wins: 255 x 257 x 255
+// 29 us; from there 301^3 float32 21 us against 35, but int32, with its scans and packing, 39 against 32,
+// and 43 against 52 at 513 x 511 x 513.
+constexpr int64_t kRepackMinPairsF32 = int64_t(1) << 24, kRepackMinPairsI32 = int64_t(1) << 26;
+
+// tropical_gemm on aligned copies of the operands that break the engine's 16-byte rules, in scratch
+// from the library's pool.  APSP_ERR_NOMEM: C is untouched (no scratch to be had, or the stream is
+// being captured into a graph, where the plain-load kernel needs none).
+static int tropical_gemm_repacked(void *C, const void *A, const void *B, int64_t M, int64_t N, int64_t K, int64_t lda,
+                                  int64_t ldb, int64_t ldc, int dtype, const void *inf, int accumulate,
+                                  cudaStream_t s) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return APSP_ERR_NOMEM;
+  }
+  auto odd = [](const void *p, int64_t ld) { return (uintptr_t)p % 16 != 0 || ld % 4 != 0; };
+  const bool ca = odd(A, lda), cb = odd(B, ldb), cc = odd(C, ldc);
+  const int64_t la = round_up(K, 4), lb = round_up(N, 4);
+  const int64_t ba = ca ? round_up(M * la * 4, 256) : 0, bb = cb ? round_up(K * lb * 4, 256) : 0;
+  const int64_t bc = cc ? round_up(M * lb * 4, 256) : 0;
+  void *own = nullptr;
+  if (ws_alloc(&own, (size_t)(ba + bb + bc), s) != APSP_OK) return APSP_ERR_NOMEM;
+  uint8_t *p = reinterpret_cast<uint8_t *>(own);
+  void *pa = p, *pb = p + ba, *pc = p + ba + bb;
+  int r = APSP_OK;
+  if (ca) r = launch_copy2d(pa, la, A, lda, M, K, s);
+  if (!r && cb) r = launch_copy2d(pb, lb, B, ldb, K, N, s);
+  if (!r && cc && accumulate) r = launch_copy2d(pc, lb, C, ldc, M, N, s);
+  if (!r)
+    r = tropical_gemm(cc ? pc : C, ca ? pa : A, cb ? pb : B, M, N, K, ca ? la : lda, cb ? lb : ldb, cc ? lb : ldc, dtype,
+                      inf, accumulate, nullptr, 0, s);
+  if (!r && cc) r = launch_copy2d(C, ldc, pc, lb, M, N, s);
+  ws_free(own, s);
+  return r;
+}
+}  // namespace apsp
+
 extern "C" size_t tropical_gemm_workspace_bytes(int64_t M, int64_t N, int64_t K, int dtype) {
   using namespace apsp;
   if (dtype != APSP_I32 || M <= 0 || N <= 0 || K <= 0) return kFlagBytes;
@@ -869,7 +909,16 @@ extern "C" int tropical_gemm(void *C, const void *A, const void *B, int64_t M, i
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const bool aligned = (uintptr_t)C % 16 == 0 && (K == 0 || ((uintptr_t)A % 16 == 0 && (uintptr_t)B % 16 == 0)) &&
                        ldc % 4 == 0 && (K == 0 || (lda % 4 == 0 && ldb % 4 == 0));
-  if (!aligned) return launch_tgemm_generic(C, A, B, M, N, K, lda, ldb, ldc, dtype, accumulate != 0, inf_i, inf_f, s);
+  if (!aligned) {
+    // Work on 16-byte aligned copies when the product is worth the passes and scratch may be taken
+    // here (no caller workspace, no capture); else the plain-load kernel.
+    const int64_t least = dtype == APSP_F32 ? kRepackMinPairsF32 : kRepackMinPairsI32;
+    if (!ws && K > 0 && M * N > least / K) {
+      const int done = tropical_gemm_repacked(C, A, B, M, N, K, lda, ldb, ldc, dtype, inf, accumulate, s);
+      if (done != APSP_ERR_NOMEM) return done;
+    }
+    return launch_tgemm_generic(C, A, B, M, N, K, lda, ldb, ldc, dtype, accumulate != 0, inf_i, inf_f, s);
+  }
   CUtensorMap mA, mB, mC;
   int r;
   if ((r = make_operand_maps(K > 0 ? A : C, K > 0 ? M : 1, K > 0 ? K : 4, K > 0 ? lda : 4, dtype, &mA, nullptr, nullptr)))

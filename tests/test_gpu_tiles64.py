@@ -121,3 +121,27 @@ def test_product(apsp, m, n, k, kind):
             want = np.minimum(want, c)
         assert_dist_equal(out.cpu().numpy(), want.astype(np.int32) if dt == np.int32 else want, f"{m}x{n}x{k} {kind}")
     assert apsp.apsp_device_status() == 0
+
+
+@pytest.mark.parametrize("dtype", ["int32", "float32"])
+@pytest.mark.parametrize("m,n,k", [(255, 257, 255), (301, 303, 305), (513, 511, 514), (640, 129, 1001)])
+def test_product_of_unaligned_operands(apsp, m, n, k, dtype):
+    """Contiguous operands whose rows are not 16-byte aligned (or only some of them): below and above the
+    sizes that run on aligned copies, with and without a caller workspace, and folded into C."""
+    rng = np.random.default_rng(m + k)
+    dt = np.dtype(dtype)
+
+    def mat(r, c):
+        v = rng.lognormal(0, 1, (r, c)) if dtype == "float32" else rng.integers(1, 1000, (r, c))
+        return np.where(rng.random((r, c)) < 0.6, v, np.inf if dtype == "float32" else INF).astype(dt)
+
+    a, b, c = mat(m, k), mat(k, n), mat(m, n)
+    A, B = torch.from_numpy(a).cuda(), torch.from_numpy(b).cuda()
+    ws = torch.empty(256, dtype=torch.uint8, device="cuda")
+    for acc in (False, True):
+        want = np.minimum(oracle.minplus(a, b), c) if acc else oracle.minplus(a, b)
+        for w in (None, ws):
+            out = torch.from_numpy(c).cuda()
+            apsp.tropical_gemm(out, A, B, accumulate=acc, ws=w)
+            assert_dist_equal(out.cpu().numpy(), want.astype(dt) if dtype == "int32" else want, f"{m}x{n}x{k} {dtype}")
+    assert apsp.apsp_device_status() == 0
