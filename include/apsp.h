@@ -276,8 +276,11 @@ int apsp_batched(void *pool, const int64_t *offsets, const int32_t *ns, const in
  * below 0x3FFFFFFF (checked on the device); otherwise a direct argmin kernel runs.  The
  * workspace (apsp_predecessors_workspace_bytes) holds the bound words and the two encoded
  * copies (2 x n x round_up(n, 4) int32).
- * float32: the direct kernel, with each sum rounded once (round to nearest) and ties to the
- * smallest k; the workspace is only the 256 bytes of bound words. */
+ * float32: each sum rounded once (round to nearest), ties to the smallest k.  From n = 128 the
+ * argmin runs on the (min,+) tiles: a product finds the 64-deep chunk of k that holds each minimum,
+ * a second pass the index in it; the workspace then holds four n x round_up(n, 4) matrices (clean
+ * copies of d, w and w transposed, and the chunks).  With a smaller workspace (256 bytes are
+ * accepted), and without one while the stream is captured, a direct kernel runs instead. */
 size_t apsp_predecessors_workspace_bytes(int64_t n, int dtype);
 int apsp_predecessors(const void *d, int64_t ldd, const void *w, int64_t ldw, int32_t *pred,
                       int64_t ldp, int64_t n, int dtype, const void *inf, void *ws,

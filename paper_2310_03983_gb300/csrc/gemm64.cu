@@ -32,7 +32,7 @@ constexpr int kSMax16 = 28;     // per stage: largest finite entry written
 constexpr int kSChanged32 = 44;
 constexpr int kSMaxStages = 16;
 
-enum { kProduct = 0, kSquare32 = 1, kSquare16 = 2 };
+enum { kProduct = 0, kSquare32 = 1, kSquare16 = 2, kArgChunk = 3 };
 
 struct G64Args {
   int M, N, K;         // K in operand words
@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(kFThreads, 1) gemm64_kernel(const __grid_const
       bool ok = true;
       for (int it = blockIdx.x * a.groups + g;; it += step, ++m) {
         int t = it, st = 0;
-        if (KIND != kProduct) {
+        if (KIND == kSquare32 || KIND == kSquare16) {
           t = atomicAdd(ctr, 1);
           st = t / a.items;
           t -= st * a.items;
@@ -139,7 +139,8 @@ __global__ void __launch_bounds__(kFThreads, 1) gemm64_kernel(const __grid_const
           slot[4 * b] = ti;
           slot[4 * b + 1] = tj;
           slot[4 * b + 2] = min(kFB, a.K - k * kFB);
-          slot[4 * b + 3] = (k == 0 ? kGFirst : 0) | (k == chunks - 1 ? kGLast : 0) | (st << kGStageShift);
+          slot[4 * b + 3] = (k == 0 ? kGFirst : 0) | (k == chunks - 1 ? kGLast : 0) |
+                            ((KIND == kArgChunk ? k : st) << kGStageShift);
           int *buf = smem + b * 2 * kFTileInts;
           mbar_arrive_expect_tx(&full[b], 2 * kFTileInts * 4);
           tma_load_2d(buf, &maps.A[set], k * kFB, ti * kFB, &full[b]);
@@ -162,7 +163,7 @@ __global__ void __launch_bounds__(kFThreads, 1) gemm64_kernel(const __grid_const
       mbar_wait(&empty[b], ((c >> 1) & 1) ^ 1, a.status);
       slot[4 * b] = -1;
       mbar_arrive(&full[b]);
-    } else if (KIND != kProduct) {  // ----------------------------- releases ----------------------
+    } else if (KIND == kSquare32 || KIND == kSquare16) {  // ------------ releases ----------------------
       for (int n = 0;; ++n) {
         const int b = n & 1;
         if (!mbar_wait(&rel_full[b], (n >> 1) & 1, a.status)) break;
@@ -181,18 +182,25 @@ __global__ void __launch_bounds__(kFThreads, 1) gemm64_kernel(const __grid_const
   const int warp = (threadIdx.x >> 5) % 4, tm = warp * 4 + (lane >> 3), tn = lane & 7;
   const bool f32 = !P16 && (a.is_float || (a.wmax && small_int_bound(a.wmax[0], a.wmult, a.wmax[1])));
   const int init = P16 ? (kCap16 << 16) | kCap16 : a.inf;
-  float acc[4][8];
+  float acc[4][8], best[KIND == kArgChunk ? 4 : 1][8];  // kArgChunk: minima so far, and the chunks
+  int arg[KIND == kArgChunk ? 4 : 1][8];                // that first reached them
   int m = 0;
   for (uint32_t c = 0;; ++c) {
     const int b = c & 1;
     if (!mbar_wait(&full[b], (c >> 1) & 1, a.status)) break;
     const int ti = slot[4 * b], tj = slot[4 * b + 1], klen = slot[4 * b + 2], flags = slot[4 * b + 3];
     if (ti < 0) break;
-    if (flags & kGFirst) {
+    if (KIND == kArgChunk || (flags & kGFirst)) {
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = __int_as_float(init);
+        for (int j = 0; j < 8; ++j) {
+          acc[i][j] = __int_as_float(init);
+          if (KIND == kArgChunk && (flags & kGFirst)) {
+            best[i][j] = __int_as_float(init);
+            arg[i][j] = -1;
+          }
+        }
     }
     const int *As = smem + b * 2 * kFTileInts, *Bs = As + kFTileInts;
     if (P16) fine_product_int<true>(As, Bs, tm, tn, klen, acc);
@@ -200,6 +208,15 @@ __global__ void __launch_bounds__(kFThreads, 1) gemm64_kernel(const __grid_const
     else fine_product_int<false>(As, Bs, tm, tn, klen, acc);
     __syncwarp();
     if (lane == 0) mbar_arrive(&empty[b]);
+    if (KIND == kArgChunk) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          arg[i][j] = acc[i][j] < best[i][j] ? flags >> kGStageShift : arg[i][j];
+          best[i][j] = fminf(best[i][j], acc[i][j]);
+        }
+    }
     if (!(flags & kGLast)) continue;
     const int ri = ti * kFB, cj = tj * kFB, set = (flags >> kGStageShift) & 1, st = flags >> kGStageShift;
     int v[4][8];
@@ -208,7 +225,8 @@ __global__ void __launch_bounds__(kFThreads, 1) gemm64_kernel(const __grid_const
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         const int x = __float_as_int(acc[i][j]);
-        if (KIND == kSquare16) v[i][j] = ArithI16x2::collapse_truncated(x);
+        if (KIND == kArgChunk) v[i][j] = arg[i][j];
+        else if (KIND == kSquare16) v[i][j] = ArithI16x2::collapse_truncated(x);
         else v[i][j] = P16 ? ArithI16x2::collapse(x, a.inf) : x;
       }
     bool diff = false;
@@ -262,8 +280,8 @@ __global__ void __launch_bounds__(kFThreads, 1) gemm64_kernel(const __grid_const
       big = __reduce_max_sync(0xffffffffu, big);
       if (lane == 0) atomicMax(a.words + kSMax16 + st, big);
     } else {
-      int *out = KIND == kProduct ? a.out[0] : a.out[set ^ 1];
-      const int64_t ldo = KIND == kProduct ? a.ldo[0] : a.ldo[set ^ 1];
+      int *out = KIND == kSquare32 ? a.out[set ^ 1] : a.out[0];
+      const int64_t ldo = KIND == kSquare32 ? a.ldo[set ^ 1] : a.ldo[0];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const int r = ri + tm + 16 * i;
@@ -282,7 +300,7 @@ __global__ void __launch_bounds__(kFThreads, 1) gemm64_kernel(const __grid_const
         }
       }
     }
-    if (KIND != kProduct) {
+    if (KIND == kSquare32 || KIND == kSquare16) {
       if (__any_sync(0xffffffffu, diff) && lane == 0) atomicOr(changed + st, 1);
       if (!mbar_wait(&rel_empty[m & 1], ((m >> 1) & 1) ^ 1, a.status)) break;
       if (warp == 0 && lane == 0) rel[m & 1] = 1;
@@ -291,7 +309,7 @@ __global__ void __launch_bounds__(kFThreads, 1) gemm64_kernel(const __grid_const
     }
     ++m;
   }
-  if (KIND != kProduct) {
+  if (KIND == kSquare32 || KIND == kSquare16) {
     mbar_wait(&rel_empty[m & 1], ((m >> 1) & 1) ^ 1, a.status);
     if (warp == 0 && lane == 0) rel[m & 1] = -1;
     __syncwarp();
@@ -457,6 +475,25 @@ int launch_gemm64(bool acc, int dtype, const void *A, int64_t lda, const void *B
   r = p.arith16 ? launch64<kProduct, true>(a, m, s) : launch64<kProduct, false>(a, m, s);
   if (tr) trace_end(s, ev, kModeGemm + p.trace_class, (double)p.M * (double)p.N * (double)p.K * (p.arith16 ? 2.0 : 1.0));
   return r;
+}
+
+int launch_arg_chunks(const float *A, int64_t lda, const float *B, int64_t ldb, int64_t n, int *out, int64_t ldo,
+                      cudaStream_t s) {
+  G64Args a = {};
+  a.M = a.N = a.K = (int)n;
+  a.tiles_n = (int)cdiv(n, kFB);
+  a.items = a.tiles_n * a.tiles_n;
+  a.stages = 1;
+  a.groups = groups_for(a.items);
+  a.is_float = 1;
+  a.inf = 0x7f800000;
+  a.out[0] = out;
+  a.ldo[0] = ldo;
+  a.status = status_word();
+  G64Maps m = {};
+  int r;
+  if ((r = maps64(&m.A[0], &m.B[0], A, n, n, lda, B, n, ldb, APSP_F32))) return r;
+  return launch64<kArgChunk, false>(a, m, s);
 }
 
 size_t squaring64_bytes(int64_t n, int dtype) {

@@ -13,6 +13,12 @@ bool gemm64_pays(int64_t M, int64_t N, int64_t K);
 int launch_gemm64(bool acc, int dtype, const void *A, int64_t lda, const void *B, int64_t ldb, const TileProblem &p,
                   cudaStream_t s);
 
+// float32, aligned n x n operands: out[i][j] = the first chunk of kArgChunkLen consecutive k that holds
+// min_k A[i][k] + B[k][j], or -1 when that minimum is +infinity.
+constexpr int kArgChunkLen = 64;
+int launch_arg_chunks(const float *A, int64_t lda, const float *B, int64_t ldb, int64_t n, int *out, int64_t ldo,
+                      cudaStream_t s);
+
 // Largest n that squaring64 takes (its stages wait on one another inside one launch; beyond it the
 // 128 x 128 tiles fill the GPU).
 constexpr int64_t kSquaring64MaxN = 4096;

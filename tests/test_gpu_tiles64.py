@@ -145,3 +145,25 @@ def test_product_of_unaligned_operands(apsp, m, n, k, dtype):
             apsp.tropical_gemm(out, A, B, accumulate=acc, ws=w)
             assert_dist_equal(out.cpu().numpy(), want.astype(dt) if dtype == "int32" else want, f"{m}x{n}x{k} {dtype}")
     assert apsp.apsp_device_status() == 0
+
+
+@pytest.mark.parametrize("ties", [False, True])
+@pytest.mark.parametrize("n", [127, 128, 129, 300, 513, 1001])
+def test_float_predecessors(apsp, n, ties):
+    """The smallest last hop, index for index, with the chunked product (from n = 128) and with the direct
+    kernel (a workspace without room for the copies); ties: half-integer weights."""
+    h = _graph(n, "f32", n + 3)
+    if ties:
+        h = np.where(np.isfinite(h), np.ceil(2 * h) / 2, h).astype(np.float32)
+        np.fill_diagonal(h, 0)
+    w = torch.from_numpy(h).cuda()
+    d = w.clone()
+    apsp.apsp_fw(d)
+    want = oracle.last_hop(d.cpu().numpy(), h, threads=THREADS)
+    full = apsp.apsp_predecessors_workspace_bytes(n, torch.float32)
+    wide = torch.full((n, n + 5), -7, dtype=torch.int32, device="cuda")  # rows of pred not 16-byte aligned
+    for ws in (None, torch.empty(256, dtype=torch.uint8, device="cuda"), torch.empty(full, dtype=torch.uint8, device="cuda")):
+        apsp.apsp_predecessors(d, w, wide[:, :n], ws=ws)
+        assert np.array_equal(wide[:, :n].cpu().numpy(), want)
+    assert torch.all(wide[:, n:] == -7)
+    assert apsp.apsp_device_status() == 0
