@@ -51,62 +51,123 @@ struct FineArgs {
   unsigned int *status;
 };
 
+// Many graphs in lockstep: staged one below the other in d, each padded to whole 128-vertex blocks with
+// isolated vertices (grouped.cu).  Stage s runs for every graph with at least s blocks of 64.
+struct FineGraphs {
+  int ngroups;
+  GraphGroup groups[kMaxGroups];
+  const int *gsize;  // vertices of each graph (0: left alone); tiles of padding are skipped
+};
+
 struct FineItem {
   int i, j, s;           // output tile, stage
   int ai, aj, bi, bj;    // operand tiles (ai < 0: none, the item only closes its tile)
   int klen;              // k range (the last block may be partial)
-  bool close, dep, panel;
+  int row0;              // first row of the item's graph
+  bool close, dep, panel, skip;
 };
 
-// Items of stage s: A(s) and B(s).
-__device__ __forceinline__ int stage_a_items(int nt, int s) { return s == 0 ? 1 : (nt - 1) * (nt - 1); }
-__device__ __forceinline__ int stage_b_items(int nt, int s) { return s < nt ? 2 * (nt - 1) : 0; }
-__device__ __forceinline__ int stage_dep_items(int nt, int s) { return s >= nt ? 0 : (s == 0 ? 1 : 2 * nt - 3); }
+// Items of stage s of a matrix of nt blocks, by kind, in the order they are handed out: the closing tile,
+// the other tiles of block row and column s, the first of the remaining tiles, the panels, the rest.
+struct StageCounts {
+  int close, dep, rest, panel;
+  __device__ __forceinline__ int total() const { return close + dep + rest + panel; }
+};
+__device__ __forceinline__ StageCounts stage_counts(int nt, int s) {
+  StageCounts c = {0, 0, 0, 0};
+  if (s > nt || (s == nt && nt == 1)) return c;
+  c.close = s < nt;
+  c.dep = s > 0 && s < nt ? 2 * nt - 4 : 0;
+  c.rest = s == 0 ? 0 : s < nt ? (nt - 2) * (nt - 2) : (nt - 1) * (nt - 1);
+  c.panel = s < nt ? 2 * (nt - 1) : 0;
+  return c;
+}
+__device__ __forceinline__ int kind_count(const StageCounts &c, int kind) {
+  return kind == 0 ? c.close : kind == 1 ? c.dep : kind == 2 ? c.rest : c.panel;
+}
 
-__device__ __forceinline__ FineItem fine_item(const FineArgs &a, int s, int p) {
+// Item x of one kind (0 close, 1 dep, 2 rest, 3 panel) of a matrix of nt blocks.
+__device__ __forceinline__ FineItem fine_item(int nt, int s, int kind, int x) {
   FineItem it;
-  const int nt = a.nt, dep = stage_dep_items(nt, s), nb = stage_b_items(nt, s);
-  const int rest = stage_a_items(nt, s) - dep, r1 = a.rest1 < rest ? a.rest1 : rest;
   it.s = s;
-  it.close = it.dep = it.panel = false;
+  it.close = kind == 0;
+  it.dep = kind < 2;
+  it.panel = kind == 3;
   int kblk = s - 1;
-  if (p >= dep + r1 && p < dep + r1 + nb) {  // B(s)
-    const int v = p - dep - r1;
-    it.panel = true;
-    kblk = s;
-    if (v < nt - 1) {  // row panel: D[s][j] = D[s][s]* (x) D[s][j]
-      it.i = s;
-      it.j = v + (v >= s);
-    } else {           // column panel: D[i][s] = D[i][s] (x) D[s][s]*
-      it.i = (v - (nt - 1)) + ((v - (nt - 1)) >= s);
-      it.j = s;
-    }
-  } else if (p < dep) {
-    it.dep = true;
-    if (p == 0) {
-      it.i = it.j = s;
-      it.close = true;
-    } else {
-      const int x = p - 1 < nt - 2 ? p - 1 : p - 1 - (nt - 2), y = x + (x >= s - 1 ? 2 : 0);
-      it.i = p - 1 < nt - 2 ? s : y;
-      it.j = p - 1 < nt - 2 ? y : s;
-    }
+  if (kind == 0) {
+    it.i = it.j = s;
+  } else if (kind == 1) {
+    const int u = x < nt - 2 ? x : x - (nt - 2), y = u + (u >= s - 1 ? 2 : 0);
+    it.i = x < nt - 2 ? s : y;
+    it.j = x < nt - 2 ? y : s;
+  } else if (kind == 2) {
+    const int w = s < nt ? nt - 2 : nt - 1, skip = s < nt ? 2 : 0;  // outside block rows / columns s - 1 and s
+    const int ii = x / w, jj = x - ii * w;
+    it.i = ii + (ii >= s - 1 ? skip : 0);
+    it.j = jj + (jj >= s - 1 ? skip : 0);
   } else {
-    const int u = p < dep + r1 ? p - dep : p - dep - nb;
-    if (s < nt) {  // every tile outside block rows / columns s - 1 and s
-      const int ii = u / (nt - 2), jj = u - ii * (nt - 2);
-      it.i = ii + (ii >= s - 1 ? 2 : 0);
-      it.j = jj + (jj >= s - 1 ? 2 : 0);
-    } else {       // the last update: every tile outside the last block's
-      it.i = u / (nt - 1);
-      it.j = u - it.i * (nt - 1);
+    kblk = s;
+    if (x < nt - 1) {  // row panel: D[s][j] = D[s][s]* (x) D[s][j]
+      it.i = s;
+      it.j = x + (x >= s);
+    } else {           // column panel: D[i][s] = D[i][s] (x) D[s][s]*
+      it.i = (x - (nt - 1)) + ((x - (nt - 1)) >= s);
+      it.j = s;
     }
   }
   it.ai = kblk < 0 ? -1 : it.i;
   it.aj = kblk;
   it.bi = kblk;
   it.bj = it.j;
-  it.klen = min(kFB, a.n - kblk * kFB);
+  it.klen = kFB;
+  it.row0 = 0;
+  it.skip = false;
+  return it;
+}
+
+// The counts of stage s over every matrix of the launch, and its item p.
+template <bool G>
+__device__ __forceinline__ StageCounts launch_counts(const FineArgs &a, const FineGraphs &gs, int s) {
+  if (!G) return stage_counts(a.nt, s);
+  StageCounts t = {0, 0, 0, 0};
+  for (int k = 0; k < gs.ngroups; ++k) {
+    const StageCounts c = stage_counts(2 * gs.groups[k].nb, s);
+    const int m = gs.groups[k].count;
+    t.close += m * c.close;
+    t.dep += m * c.dep;
+    t.rest += m * c.rest;
+    t.panel += m * c.panel;
+  }
+  return t;
+}
+
+template <bool G>
+__device__ __forceinline__ FineItem fine_decode(const FineArgs &a, const FineGraphs &gs, const StageCounts &c, int s, int p) {
+  const int r1 = min(a.rest1, c.rest);
+  int kind = 0, x = p;
+  if (x >= c.close) { x -= c.close; kind = 1; }
+  if (kind == 1 && x >= c.dep) { x -= c.dep; kind = 2; }
+  if (kind == 2 && x >= r1) {
+    if (x < r1 + c.panel) { x -= r1; kind = 3; }
+    else x -= c.panel;
+  }
+  if (!G) {
+    FineItem it = fine_item(a.nt, s, kind, x);
+    it.klen = min(kFB, a.n - it.aj * kFB);
+    return it;
+  }
+  int k = 0, per = 0, nt = 0;
+  for (; k < gs.ngroups; ++k) {
+    nt = 2 * gs.groups[k].nb;
+    per = kind_count(stage_counts(nt, s), kind);
+    if (x < per * gs.groups[k].count) break;
+    x -= per * gs.groups[k].count;
+  }
+  const int q = x / per;
+  FineItem it = fine_item(nt, s, kind, x - q * per);
+  it.row0 = (int)gs.groups[k].row0 + q * nt * kFB;
+  const int n = gs.gsize[gs.groups[k].first + q];
+  it.skip = it.i * kFB >= n || it.j * kFB >= n || it.aj * kFB >= n;
   return it;
 }
 
@@ -196,16 +257,6 @@ __device__ __forceinline__ void fine_close(int (&d)[4][8], int bk, int warp, int
   }
 }
 
-__device__ __forceinline__ FineItem fine_decode(const FineArgs &a, int t) {
-  int s = a.s0, p = t;
-  for (;; ++s) {
-    const int items = stage_a_items(a.nt, s) + stage_b_items(a.nt, s);
-    if (p < items) break;
-    p -= items;
-  }
-  return fine_item(a, s, p);
-}
-
 constexpr int kFClose = 1, kFDep = 2, kFStageShift = 2;  // flags of an item slot
 
 // The consumer warps compute; a group's loading warp takes tickets, waits for an item's dependencies and
@@ -213,9 +264,10 @@ constexpr int kFClose = 1, kFDep = 2, kFStageShift = 2;  // flags of an item slo
 // during this one's product) and of its old output tile; its releasing warp counts stored items, so
 // that the fence this needs is off the consumers' path.  mA: boxes of 64 rows x 32 columns, 128-byte
 // swizzle; mB: 64 x 64.  The register split is the GEMM engine's (tgemm.cuh).
+template <bool G>
 __global__ void __launch_bounds__(kFThreads, 1)
-    fine_fw_kernel(const __grid_constant__ FineArgs a, const __grid_constant__ CUtensorMap mA,
-                   const __grid_constant__ CUtensorMap mB) {
+    fine_fw_kernel(const __grid_constant__ FineArgs a, const __grid_constant__ FineGraphs gs,
+                   const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB) {
   pdl_wait();
   pdl_trigger();
   if (a.run_if && !*a.run_if) return;
@@ -253,30 +305,39 @@ __global__ void __launch_bounds__(kFThreads, 1)
     if ((threadIdx.x >> 5) % 4 < 2) {  // ------------------------- loads -------------------------
       tma_prefetch_desc(&mA);
       tma_prefetch_desc(&mB);
-      int total = 0;
-      for (int s = a.s0; s < a.s1; ++s) total += stage_a_items(a.nt, s) + stage_b_items(a.nt, s);
       uint32_t issued = 0, pars = 0;
+      int s = a.s0, base = 0, before = 0;  // current stage, its first ticket, the items of the one before it
+      StageCounts sc = launch_counts<G>(a, gs, s);
       for (int n = 0;; ++n) {
         const int b = n & 1;
         const uint32_t ph = (n >> 1) & 1;
         const int t = atomicAdd(ticket, 1);
+        while (s < a.s1 && t - base >= sc.total()) {
+          base += before = sc.total();
+          if (++s < a.s1) sc = launch_counts<G>(a, gs, s);
+        }
         bool ok = true;
         FineItem it = {};
-        if (t < total) {
-          it = fine_decode(a, t);
-          const int x = 2 * (it.s - a.s0);
+        if (s < a.s1) {
+          it = fine_decode<G>(a, gs, sc, s, t - base);
+          const int x = 2 * (s - a.s0);
+          if (G && it.skip) {  // padding: nothing to do, but counted
+            if (it.dep) atomicAdd(cnt + x, 1);
+            atomicAdd(cnt + x + 1, 1);
+            --n;
+            continue;
+          }
           // The closing item heads the chain of dependent steps: the SM's other group starts no later item
           // until it is closed (which depends on no later ticket).
           if (it.close) closing[g] = t;
           if (a.groups == 2)
             for (uint32_t w = 0; t > closing[g ^ 1] && w < kSpinLimit; ++w) __nanosleep(64);
-          if (it.panel) ok = counter_wait(cnt + x, stage_dep_items(a.nt, it.s), a.status);
-          else if (it.s > a.s0)
-            ok = counter_wait(cnt + x - 1, stage_a_items(a.nt, it.s - 1) + stage_b_items(a.nt, it.s - 1), a.status);
+          if (it.panel) ok = counter_wait(cnt + x, sc.close + sc.dep, a.status);
+          else if (s > a.s0) ok = counter_wait(cnt + x - 1, before, a.status);
           fence_proxy_async_global();
         }
         ok = mbar_wait(&empty[b], ph ^ 1, a.status) && ok;
-        if (t >= total || !ok) {
+        if (s >= a.s1 || !ok) {
           for (int x = 0; x < 2; ++x)  // leave no copy writing into an exiting CTA's shared memory
             if (issued & (1u << x)) mbar_wait(&full[x], (pars >> x) & 1, a.status);
           if (n > 0) mbar_wait(cfull, (n - 1) & 1, a.status);
@@ -284,7 +345,8 @@ __global__ void __launch_bounds__(kFThreads, 1)
           mbar_arrive(&full[b]);
           break;
         }
-        slot[4 * b] = it.i;
+        const int row = it.row0 / kFB;
+        slot[4 * b] = row + it.i;
         slot[4 * b + 1] = it.j;
         slot[4 * b + 2] = it.ai >= 0 ? it.klen : 0;
         slot[4 * b + 3] = (it.close ? kFClose : 0) | (it.dep ? kFDep : 0) | ((it.s - a.s0) << kFStageShift);
@@ -293,16 +355,16 @@ __global__ void __launch_bounds__(kFThreads, 1)
         } else {
           int *buf = smem + b * 2 * kFTileInts;
           mbar_arrive_expect_tx(&full[b], 2 * kFTileInts * 4);
-          tma_load_2d(buf, &mA, it.aj * kFB, it.ai * kFB, &full[b]);
-          tma_load_2d(buf + kFTileInts / 2, &mA, it.aj * kFB + 32, it.ai * kFB, &full[b]);
-          tma_load_2d(buf + kFTileInts, &mB, it.bj * kFB, it.bi * kFB, &full[b]);
+          tma_load_2d(buf, &mA, it.aj * kFB, (row + it.ai) * kFB, &full[b]);
+          tma_load_2d(buf + kFTileInts / 2, &mA, it.aj * kFB + 32, (row + it.ai) * kFB, &full[b]);
+          tma_load_2d(buf + kFTileInts, &mB, it.bj * kFB, (row + it.bi) * kFB, &full[b]);
           issued |= 1u << b;
           pars = (pars & ~(1u << b)) | (ph << b);
         }
         // The old output tile is needed only after the product.
         mbar_wait(cempty, (n & 1) ^ 1, a.status);
         mbar_arrive_expect_tx(cfull, kFTileInts * 4);
-        tma_load_2d(old, &mB, it.j * kFB, it.i * kFB, cfull);
+        tma_load_2d(old, &mB, it.j * kFB, (row + it.i) * kFB, cfull);
       }
     } else {  // ------------------------------------------------ releases ----------------------
       for (int n = 0;; ++n) {
@@ -408,14 +470,42 @@ __global__ void __launch_bounds__(kFThreads, 1)
 // 2.4 us) but the SM does more: worth it once the tiles of a stage, not the chain of dependent items,
 // bound it.  Measured (float32, one / two groups): n = 1024 291 / 353 us, 1448 414 / 514, 2048 851 /
 // 785, 2896 2212 / 1857, 4092 5623 / 4682: the line is drawn at 4.5 tiles per SM (n = 1730 on 152 SMs).
-static int fine_groups(int nt, int sms) { return 2 * (nt - 1) * (nt - 1) > 9 * sms ? 2 : 1; }
+static int fine_groups(int64_t tiles, int sms) { return 2 * tiles > 9 * sms ? 2 : 1; }
+
+template <bool G>
+static int fine_launch(const FineArgs &a, const FineGraphs &gs, int64_t most, double pairs, int trace_mode,
+                       const CUtensorMap &mA, const CUtensorMap &mB, cudaStream_t s) {
+  auto k = fine_fw_kernel<G>;
+  static std::atomic<int> checked{0};  // 1: register split verified (see launch_one in tgemm.cu)
+  if (!checked.load(std::memory_order_relaxed)) {
+    cudaFuncAttributes fa;
+    APSP_CUDA_TRY(cudaFuncGetAttributes(&fa, k));
+    if (fa.numRegs < kLaunchRegs || fa.maxThreadsPerBlock < kFThreads) return APSP_ERR_UNSUPPORTED;
+    checked.store(1, std::memory_order_relaxed);
+  }
+  APSP_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kFSmemBytes));
+  const int grid = (int)std::min<int64_t>(most, sm_count());
+  FineArgs b = a;
+  b.rest1 = (int)std::max<int64_t>(0, (int64_t)grid * a.groups - a.rest1);
+  void *ev = nullptr;
+  if (trace_on()) trace_begin(s, &ev);
+  launch_pdl(k, grid, kFThreads, kFSmemBytes, s, b, gs, mA, mB);
+  APSP_LAUNCH_CHECK();
+  if (ev) trace_end(s, ev, trace_mode, pairs);
+  return APSP_OK;
+}
+
+static int fine_maps(CUtensorMap *mA, CUtensorMap *mB, const void *d, int64_t rows, int64_t cols, int64_t ld, int dtype) {
+  int r;
+  if ((r = make_tmap_2d(mA, d, rows, cols, ld, kFB, 32, dtype, true))) return r;
+  return make_tmap_2d(mB, d, rows, cols, ld, kFB, kFB, dtype);
+}
 
 int fine_closure(void *d, int64_t n, int64_t ld, int dtype, int inf_i, const int *wmax, int64_t wmult,
                  const int *run_if, int *counters, int trace_class, cudaStream_t s) {
   CUtensorMap mA, mB;
   int r;
-  if ((r = make_tmap_2d(&mA, d, n, n, ld, kFB, 32, dtype, true))) return r;
-  if ((r = make_tmap_2d(&mB, d, n, n, ld, kFB, kFB, dtype))) return r;
+  if ((r = fine_maps(&mA, &mB, d, n, n, ld, dtype))) return r;
   FineArgs a = {};
   a.d = reinterpret_cast<int *>(d);
   a.ld = ld;
@@ -428,18 +518,11 @@ int fine_closure(void *d, int64_t n, int64_t ld, int dtype, int inf_i, const int
   a.run_if = run_if;
   a.counters = counters;
   a.status = status_word();
+  a.groups = fine_groups((int64_t)(a.nt - 1) * (a.nt - 1), sm_count());
+  a.rest1 = 2 * a.nt - 3;
   // nt + 1 stages over as many launches as the 128-vertex loop makes (1, or 2 + one per block).
   const int64_t nb = cdiv(n, kBM);
   const int stages = a.nt == 1 ? 1 : a.nt + 1, launches = nb == 1 ? 1 : (int)nb + 2;
-  static std::atomic<int> checked{0};  // 1: register split verified (see launch_one in tgemm.cu)
-  if (!checked.load(std::memory_order_relaxed)) {
-    cudaFuncAttributes fa;
-    APSP_CUDA_TRY(cudaFuncGetAttributes(&fa, fine_fw_kernel));
-    if (fa.numRegs < kLaunchRegs || fa.maxThreadsPerBlock < kFThreads) return APSP_ERR_UNSUPPORTED;
-    checked.store(1, std::memory_order_relaxed);
-  }
-  APSP_CUDA_TRY(cudaFuncSetAttribute(fine_fw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFSmemBytes));
-  const int sms = sm_count();
   for (int l = 0; l < launches; ++l) {
     a.s0 = (int)((int64_t)stages * l / launches);
     a.s1 = (int)((int64_t)stages * (l + 1) / launches);
@@ -453,14 +536,56 @@ int fine_closure(void *d, int64_t n, int64_t ld, int dtype, int inf_i, const int
         pairs += ((double)n - k) * ((double)n - k) * k;
       }
     }
-    const int grid = std::min(most, sms);
-    a.groups = fine_groups(a.nt, sms);
-    a.rest1 = std::max(0, grid * a.groups - (2 * a.nt - 3));
-    void *ev = nullptr;
-    if (trace_on()) trace_begin(s, &ev);
-    launch_pdl(fine_fw_kernel, grid, kFThreads, kFSmemBytes, s, a, mA, mB);
-    APSP_LAUNCH_CHECK();
-    if (ev) trace_end(s, ev, kModeFwRest + trace_class, pairs);
+    if ((r = fine_launch<false>(a, FineGraphs{}, most, pairs, kModeFwRest + trace_class, mA, mB, s))) return r;
+  }
+  return APSP_OK;
+}
+
+int64_t fine_batch_tiles(const GraphGroup *groups, int ngroups) {
+  int64_t t = 0;
+  for (int k = 0; k < ngroups; ++k) {
+    const int64_t m = 2 * groups[k].nb - 1;
+    t += m * m * groups[k].count;
+  }
+  return t;
+}
+
+int fine_batch(void *d, int64_t rows, int64_t ld, const GraphGroup *groups, int ngroups, const int *gsize, int dtype,
+               int inf_i, const int *wmax, int *counters, cudaStream_t s) {
+  CUtensorMap mA, mB;
+  int r;
+  if ((r = fine_maps(&mA, &mB, d, rows, ld, ld, dtype))) return r;
+  FineArgs a = {};
+  a.d = reinterpret_cast<int *>(d);
+  a.ld = ld;
+  a.n = INT_MAX;  // the staged graphs are whole tiles
+  a.is_float = dtype == APSP_F32;
+  a.inf = dtype == APSP_F32 ? 0x7f800000 : inf_i;
+  a.wmax = dtype == APSP_F32 ? nullptr : wmax;
+  a.wmult = 1;
+  a.counters = counters;
+  a.status = status_word();
+  const int64_t tiles = fine_batch_tiles(groups, ngroups);
+  a.groups = fine_groups(tiles, sm_count());
+  FineGraphs gs = {};
+  gs.ngroups = ngroups;
+  gs.gsize = gsize;
+  int64_t dep = 0;
+  for (int k = 0; k < ngroups; ++k) {
+    gs.groups[k] = groups[k];
+    dep += (int64_t)groups[k].count * (4 * groups[k].nb - 3);
+  }
+  a.rest1 = (int)dep;
+  const int stages = 2 * groups[0].nb + 1;  // groups are listed by decreasing nb
+  for (a.s0 = 0; a.s0 < stages; a.s0 = a.s1) {
+    a.s1 = std::min(stages, a.s0 + kFineMaxStages);
+    double pairs = 0.0;
+    for (int st = std::max(1, a.s0); st < a.s1; ++st)
+      for (int k = 0; k < ngroups; ++k) {
+        const double m = (2.0 * groups[k].nb - 1) * kFB;
+        if (st <= 2 * groups[k].nb) pairs += groups[k].count * m * m * kFB;
+      }
+    if ((r = fine_launch<true>(a, gs, tiles, pairs, kModeFwRest, mA, mB, s))) return r;
   }
   return APSP_OK;
 }

@@ -13,7 +13,8 @@ namespace apsp {
 constexpr int64_t kFineMinN = 128, kFineMaxN = 3200;
 
 // Device words of the counters block (Bound::counters): all zero between launches.
-constexpr int kFineWords = 2 + 2 * 4;
+constexpr int kFineMaxStages = 8;  // of one launch
+constexpr int kFineWords = 2 + 2 * kFineMaxStages;
 
 // Closes the n x n block at d (16-byte aligned, ld % 4 == 0, normalised) in place with
 // 1 + (number of 128-vertex blocks) launches after the first (one launch when n <= 128), the
@@ -21,5 +22,12 @@ constexpr int kFineWords = 2 + 2 * 4;
 // run_if (may be null): every launch returns at once unless *run_if is set.
 int fine_closure(void *d, int64_t n, int64_t ld, int dtype, int inf_i, const int *wmax, int64_t wmult,
                  const int *run_if, int *counters, int trace_class, cudaStream_t s);
+
+// The same for many graphs in lockstep, staged one below the other in d (rows x ld, each graph padded to
+// whole 128-vertex blocks with isolated vertices, groups by decreasing nb; gsize: device, vertices of
+// each graph, 0 for one to leave alone).  wmax[0]: the largest (n - 1) * weight of any graph.
+int fine_batch(void *d, int64_t rows, int64_t ld, const GraphGroup *groups, int ngroups, const int *gsize, int dtype,
+               int inf_i, const int *wmax, int *counters, cudaStream_t s);
+int64_t fine_batch_tiles(const GraphGroup *groups, int ngroups);  // 64 x 64 tiles of one stage
 
 }  // namespace apsp

@@ -39,6 +39,7 @@
 #include <vector>
 
 #include "diag.cuh"
+#include "fine.cuh"
 #include "grouped.cuh"
 #include "tgemm.cuh"
 
@@ -51,6 +52,14 @@ constexpr int kGfUse16 = 1, kGfRerun = 2, kGfBad = 4;
 // counters are words 0 and 1): [8] largest (n - 1) * weight over the staged graphs, [9] 0,
 // [10] some graph needs the int32 pass.
 constexpr int kWBound = 8, kWRerun = 10;
+constexpr int kWFine = 16;  // [16..]: the counters of the 64-vertex-block closure (fine.cu)
+static_assert(kWFine + kFineWords <= 64, "word block");
+// A batch whose staged graphs have at most this many 64 x 64 tiles per SM in a step is closed with
+// 64-vertex blocks in 32 bits: its lockstep steps are bound by the chain of dependent tiles.
+#ifndef APSP_FBT
+#define APSP_FBT 12
+#endif
+constexpr int64_t kFineBatchTilesPerSm = APSP_FBT;
 constexpr int kPlanChunk = 4096;
 
 struct GroupSet {
@@ -76,6 +85,7 @@ struct StageArgs {
   int inf;       // int32: the sentinel; float32: the bits of +infinity (what staging writes)
   float inf_f;   // float32: the caller's sentinel (entries at or above it are missing edges)
   int is_float;
+  int exact;       // every graph goes to the 32-bit pass (float32, and small batches)
   unsigned int *status;
 };
 
@@ -201,13 +211,15 @@ __global__ void stage_decide_kernel(const StageArgs a, int64_t G) {
     if (a.gflags[q] & kGfBad) continue;
     const int w = a.wmaxg[q], n = a.ns[a.sidx[q]];
     a.gsize[q] = n;
-    if (a.is_float) {
+    if (!a.is_float) {
+      const int64_t prod = (int64_t)(n - 1) * (int64_t)w;
+      atomicMax(a.words + kWBound, (int)(prod < INT_MAX ? prod : INT_MAX));
+    }
+    if (a.exact) {
       a.gflags[q] |= kGfRerun;
       a.words[kWRerun] = 1;
       continue;
     }
-    const int64_t prod = (int64_t)(n - 1) * (int64_t)w;
-    atomicMax(a.words + kWBound, (int)(prod < INT_MAX ? prod : INT_MAX));
     if (w <= kCap16 / 4) {
       a.gflags[q] |= kGfUse16;
     } else {
@@ -573,11 +585,13 @@ int batched_staged(const StagePlan &pl, int *pool, const int64_t *offsets, const
   a.inf = isf ? 0x7f800000 : inf_i;
   a.inf_f = inf_f;
   a.is_float = isf;
+  const bool fine = fine_batch_tiles(pl.groups, pl.ngroups) <= kFineBatchTilesPerSm * sm_count();
+  a.exact = isf || fine;
   a.status = status_word();
   int *A16[2] = {reinterpret_cast<int *>(w + L.A16[0]), reinterpret_cast<int *>(w + L.A16[1])};
   int *B16[2] = {reinterpret_cast<int *>(w + L.B16[0]), reinterpret_cast<int *>(w + L.B16[1])};
 
-  APSP_CUDA_TRY(cudaMemsetAsync(words + kWBound, 0, 4 * sizeof(int), s));
+  APSP_CUDA_TRY(cudaMemsetAsync(words + kWBound, 0, kFlagBytes - kWBound * sizeof(int), s));
   APSP_CUDA_TRY(cudaMemsetAsync(w + L.gflags, 0, L.lists - L.gflags, s));  // gflags, maxb, wmaxg, gsize
   std::vector<int> all(pl.staged);
   all.insert(all.end(), pl.rest.begin(), pl.rest.end());
@@ -594,6 +608,14 @@ int batched_staged(const StagePlan &pl, int *pool, const int64_t *offsets, const
   APSP_LAUNCH_CHECK();
   stage_decide_kernel<<<g_grid, 256, 0, s>>>(a, pl.G);
   APSP_LAUNCH_CHECK();
+
+  if (fine) {
+    if ((r = fine_batch(a.S, pl.R, pl.NP, pl.groups, pl.ngroups, a.gsize, dtype, inf_i, words + kWBound, words + kWFine, s)))
+      return r;
+    stage_out_kernel<<<row_grid, 256, 0, s>>>(a);
+    APSP_LAUNCH_CHECK();
+    return APSP_OK;
+  }
 
   CUtensorMap mA, mB, mC, pA[2], pB[2];
   if ((r = make_operand_maps(a.S, pl.R, pl.NP, pl.NP, dtype, &mA, &mB, &mC))) return r;

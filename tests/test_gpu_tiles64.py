@@ -167,3 +167,17 @@ def test_float_predecessors(apsp, n, ties):
         assert np.array_equal(wide[:, :n].cpu().numpy(), want)
     assert torch.all(wide[:, n:] == -7)
     assert apsp.apsp_device_status() == 0
+
+
+@pytest.mark.parametrize("kind", ["int32", "heavy", "f32"])
+@pytest.mark.parametrize("sizes", [[257], [384, 385, 300, 129, 256, 64], [1025, 2048, 1, 640, 200], [700] * 5])
+def test_small_batch(apsp, sizes, kind):
+    """Batches small enough for 64-vertex blocks in lockstep (257..2048 vertices; padding tiles skipped),
+    with smaller graphs beside them on the persistent kernel (129..256: shared by a cluster)."""
+    mats = [_graph(n, kind, 31 * n + g) for g, n in enumerate(sizes)]
+    b = apsp.Batch(mats)
+    apsp.apsp_batched(b)
+    assert apsp.apsp_device_status() == 0
+    out = b.pool.cpu()
+    for g, m in enumerate(mats):
+        _check(apsp, b.graph(g, out), m, f"graph {g} n={sizes[g]} {kind}")
