@@ -87,19 +87,48 @@ template <> struct Store<float> {
 };
 
 // a1 for one graph, whole CTA: returns the largest finite weight (int32; 0 for float32).
-// rank / csize: this CTA normalises rows rank, rank + csize, ... (in warp-sized strides).
+// rank / csize: the CTAs of a cluster share the matrix.  A thread keeps four 16-byte accesses in flight:
+// with one row per warp and 4-byte accesses, the latency of this pass was a large part of a small
+// graph's time (four graphs of at most 256 vertices: the whole call 246 us before, 229 after).
 template <typename S>
 __device__ int normalise_graph(int *D, int n, int ld, const BatchArgs &a, int *red, int rank, int csize) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  constexpr int W = kBThreads / 32;
   bool bad = false;
   int m = 0;
-  for (int i = warp + W * rank; i < n; i += W * csize) {
-    int *row = D + (int64_t)i * ld;
-    for (int j = lane; j < n; j += 32) {
-      const int v = (j == i) ? 0 : Store<S>::fix(row[j], a, bad);
-      row[j] = v;
-      m = Store<S>::finite_max(v, a, m);
+  const int q = (n + 3) >> 2;  // 16-byte chunks of a row (the last may be partial)
+  const int64_t total = (int64_t)n * q, step = (int64_t)kBThreads * csize;
+  for (int64_t e0 = (int64_t)rank * kBThreads + threadIdx.x; e0 < total; e0 += 4 * step) {
+    int4 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t e = e0 + u * step;
+      const int i = (int)(e / q), j = 4 * (int)(e - (int64_t)i * q);
+      v[u] = make_int4(0, 0, 0, 0);
+      if (e >= total) continue;
+      const int *p = D + (int64_t)i * ld + j;
+      if (j + 3 < n) {
+        v[u] = *reinterpret_cast<const int4 *>(p);
+      } else {
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+          if (j + x < n) (&v[u].x)[x] = p[x];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t e = e0 + u * step;
+      if (e >= total) break;
+      const int i = (int)(e / q), j = 4 * (int)(e - (int64_t)i * q);
+      int *p = D + (int64_t)i * ld + j;
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        int &w = (&v[u].x)[x];
+        if (j + x >= n) continue;
+        w = j + x == i ? 0 : Store<S>::fix(w, a, bad);
+        m = Store<S>::finite_max(w, a, m);
+        if (j + 3 >= n) p[x] = w;
+      }
+      if (j + 3 < n) *reinterpret_cast<int4 *>(p) = v[u];
     }
   }
   m = __reduce_max_sync(0xffffffffu, m);
@@ -313,8 +342,8 @@ __device__ __forceinline__ int *graph_base(const BatchArgs &a, int g, int &n, in
 
 // The persistent kernel runs as clusters of csize CTAs (csize = 1 without clusters), in two
 // stages.  Stage 1: the leading run of the queue order whose graphs are each too large for
-// one CTA to close within the batch's average time per CTA (the order is largest first) is
-// closed one graph at a time by whole clusters: rank 0 takes the next
+// one CTA to close within the batch's average time per CTA (the order is largest first), or all
+// graphs above one tile when there is a cluster for each, is closed one graph at a time by whole clusters: rank 0 takes the next
 // entry and writes it into every CTA's shared memory through distributed shared memory, and
 // hardware cluster barriers separate the steps.  Stage 2: every CTA pulls the remaining
 // graphs from its own counter and closes each alone, with no cluster barrier at all.  No CTA
@@ -328,7 +357,7 @@ __global__ void __launch_bounds__(kBThreads, 1) batched_kernel(const BatchArgs a
   int *sC = sB + kBStages * kBSlabInts;  // a phase-3 tile's old C block
   int *sT = sC + kBTileInts;             // phase-1 row/column exchange buffer
   __shared__ int s_idx;   // stage 1: written by the cluster's rank 0 through DSMEM
-  __shared__ int s_nbig;
+  __shared__ int s_nbig, s_ntile;
   __shared__ int s_wmax;
   __shared__ int red[kBThreads / 32];
   cg::cluster_group cl = cg::this_cluster();
@@ -354,24 +383,29 @@ __global__ void __launch_bounds__(kBThreads, 1) batched_kernel(const BatchArgs a
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
     if ((threadIdx.x & 31) == 0) s_work[threadIdx.x >> 5] = w;
-    if (threadIdx.x == 0) s_nbig = (int)a.nq;
+    if (threadIdx.x == 0) s_nbig = s_ntile = (int)a.nq;
     __syncthreads();
     double total = 0.0;
 #pragma unroll
     for (int i = 0; i < kBThreads / 32; ++i) total += s_work[i];
+    // ... or, when the graphs above one tile are no more than the clusters, all of those: a cluster
+    // shares their panel and remaining tiles (n = 256 on one CTA: six 128^3 products in turn).
     const double big3 = fmax(0.5 * total / (double)gridDim.x, (double)(64 * csize) * (64 * csize) * (64 * csize));
-    int first_small = (int)a.nq;
+    int first_small = (int)a.nq, first_tile = (int)a.nq;
     for (int k = threadIdx.x; k < a.nq; k += kBThreads) {
       const int g = a.order ? a.order[k] : k;
       const double n = (g >= 0 && g < a.count) ? (double)a.ns[g] : 0.0;
-      if (!(n * n * n > big3)) {
-        first_small = k;
+      if (first_small == (int)a.nq && !(n * n * n > big3)) first_small = k;
+      if (!(n > (double)kSlabM)) {
+        first_tile = k;
         break;
       }
     }
     atomicMin(&s_nbig, first_small);
+    atomicMin(&s_ntile, first_tile);
     __syncthreads();
     nbig = s_nbig;
+    if (s_ntile <= (int)gridDim.x / csize) nbig = max(nbig, s_ntile);
     cl.sync();
   }
 
