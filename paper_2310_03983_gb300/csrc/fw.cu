@@ -162,13 +162,29 @@ __global__ void __launch_bounds__(256) trunc_certify_kernel(int *d, int64_t ld, 
   const int cap = cap_in_use(words);
   if (!cap) return;
   int m = 0;
-  for (int64_t i = blockIdx.x; i < n; i += gridDim.x)
-    for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
-      int *e = d + i * ld + j;
-      const int v = *e;
-      if (v < cap) m = max(m, v);
-      else if (v != inf) *e = inf;
+  for (int64_t i = blockIdx.x; i < n; i += gridDim.x) {
+    int *row = d + i * ld;  // 16-byte aligned
+    for (int64_t v = threadIdx.x; v < (n >> 2); v += blockDim.x) {
+      int4 *p = reinterpret_cast<int4 *>(row) + v;
+      int4 r = *p;
+      bool changed = false;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        int &x = (&r.x)[q];
+        if (x < cap) m = max(m, x);
+        else if (x != inf) {
+          x = inf;
+          changed = true;
+        }
+      }
+      if (changed) *p = r;
     }
+    for (int64_t j = (n & ~int64_t(3)) + threadIdx.x; j < n; j += blockDim.x) {
+      const int v = row[j];
+      if (v < cap) m = max(m, v);
+      else if (v != inf) row[j] = inf;
+    }
+  }
   m = __reduce_max_sync(0xffffffffu, m);
   if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(words + 5, m);
 }

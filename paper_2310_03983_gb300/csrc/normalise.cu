@@ -30,6 +30,8 @@ template <> __device__ __forceinline__ int finite_max<int>(int v, int inf, int m
 template <typename T>
 __global__ void __launch_bounds__(256) normalise_kernel(T *d, int64_t n, int64_t ld, T inf, bool vec, unsigned int *st,
                                                         int *wmax) {
+  pdl_wait();
+  pdl_trigger();
   bool bad = false;
   int m = 0;
   for (int64_t i = blockIdx.x; i < n; i += gridDim.x) {
@@ -62,14 +64,25 @@ __global__ void __launch_bounds__(256) normalise_kernel(T *d, int64_t n, int64_t
   if (__syncthreads_or(bad) && threadIdx.x == 0) flag_status(st, APSP_ERR_DOMAIN);
 }
 
+// vec: rows are 16-byte aligned.
 __global__ void __launch_bounds__(256) scan_max_kernel(const int *x, int64_t rows, int64_t cols, int64_t ld, int inf,
-                                                       int *out) {
+                                                       bool vec, int *out) {
+  pdl_wait();
+  pdl_trigger();
   int m = 0;
-  for (int64_t i = blockIdx.x; i < rows; i += gridDim.x)
-    for (int64_t j = threadIdx.x; j < cols; j += blockDim.x) {
-      const int v = x[i * ld + j];
-      if (v < inf) m = max(m, v);
+  for (int64_t i = blockIdx.x; i < rows; i += gridDim.x) {
+    const int *row = x + i * ld;
+    int64_t j0 = 0;
+    if (vec) {
+      const int64_t nv = cols >> 2;
+      for (int64_t v = threadIdx.x; v < nv; v += blockDim.x) {
+        const int4 r = reinterpret_cast<const int4 *>(row)[v];
+        m = finite_max(r.x, inf, finite_max(r.y, inf, finite_max(r.z, inf, finite_max(r.w, inf, m))));
+      }
+      j0 = nv << 2;
     }
+    for (int64_t j = j0 + threadIdx.x; j < cols; j += blockDim.x) m = finite_max(row[j], inf, m);
+  }
   m = __reduce_max_sync(0xffffffffu, m);
   if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(out, m);
 }
@@ -77,8 +90,9 @@ __global__ void __launch_bounds__(256) scan_max_kernel(const int *x, int64_t row
 int launch_scan_max(const void *x, int64_t rows, int64_t cols, int64_t ld, int inf, int *out, cudaStream_t s) {
   if (rows == 0 || cols == 0) return APSP_OK;
   const int64_t cap = (int64_t)sm_count() * 8;
-  scan_max_kernel<<<(int)(rows < cap ? rows : cap), 256, 0, s>>>(reinterpret_cast<const int *>(x), rows, cols, ld,
-                                                                 inf, out);
+  const bool vec = reinterpret_cast<uintptr_t>(x) % 16 == 0 && ld % 4 == 0;
+  launch_pdl(scan_max_kernel, (int)(rows < cap ? rows : cap), 256, 0, s, reinterpret_cast<const int *>(x), rows, cols,
+             ld, inf, vec, out);
   APSP_LAUNCH_CHECK();
   return APSP_OK;
 }
@@ -89,9 +103,10 @@ int launch_normalise(void *d, int64_t n, int64_t ld, int dtype, int inf_i, float
   const int64_t cap = (int64_t)sm_count() * 8;
   const int grid = (int)(n < cap ? n : cap);
   if (dtype == APSP_I32)
-    normalise_kernel<int><<<grid, 256, 0, s>>>(reinterpret_cast<int *>(d), n, ld, inf_i, vec, status_word(), wmax);
+    launch_pdl(normalise_kernel<int>, grid, 256, 0, s, reinterpret_cast<int *>(d), n, ld, inf_i, vec, status_word(), wmax);
   else
-    normalise_kernel<float><<<grid, 256, 0, s>>>(reinterpret_cast<float *>(d), n, ld, inf_f, vec, status_word(), nullptr);
+    launch_pdl(normalise_kernel<float>, grid, 256, 0, s, reinterpret_cast<float *>(d), n, ld, inf_f, vec, status_word(),
+               nullptr);
   APSP_LAUNCH_CHECK();
   return APSP_OK;
 }

@@ -677,6 +677,7 @@ __device__ __forceinline__ bool fits16(const int *words) {
   return (int64_t)words[0] + (int64_t)words[1] < kCap16;
 }
 __device__ __forceinline__ int cap16(int v, int inf) { return v >= inf ? kCap16 : v; }
+// The operands' rows are 16-byte aligned (the engine's own condition).
 
 __global__ void __launch_bounds__(256) pack16_a_kernel(const int *A, int64_t lda, int64_t M, int64_t K, int *A16,
                                                        int64_t ld16, int inf, int *words) {
@@ -688,7 +689,14 @@ __global__ void __launch_bounds__(256) pack16_a_kernel(const int *A, int64_t lda
   for (int64_t i = blockIdx.x; i < M; i += gridDim.x) {
     const int *ar = A + i * lda;
     int *o = A16 + i * ld16;
-    for (int64_t w = threadIdx.x; w < kw; w += blockDim.x) {
+    // Two words per thread from one 16-byte load (rows of A are 16-byte aligned, of A16 too).
+    const int64_t nv = K >> 2;
+    for (int64_t v = threadIdx.x; v < nv; v += blockDim.x) {
+      const int4 r = reinterpret_cast<const int4 *>(ar)[v];
+      reinterpret_cast<int2 *>(o)[v] = make_int2((cap16(r.y, inf) << 16) | cap16(r.x, inf),
+                                                 (cap16(r.w, inf) << 16) | cap16(r.z, inf));
+    }
+    for (int64_t w = 2 * nv + threadIdx.x; w < kw; w += blockDim.x) {
       const int64_t k = 2 * w;
       const int lo = cap16(ar[k], inf), hi = k + 1 < K ? cap16(ar[k + 1], inf) : kCap16;
       o[w] = (hi << 16) | lo;
@@ -707,7 +715,14 @@ __global__ void __launch_bounds__(256) pack16_b_kernel(const int *B, int64_t ldb
     const int *r0 = B + 2 * w * ldb, *r1 = r0 + ldb;
     const bool has1 = 2 * w + 1 < K;
     int *o = B16 + w * ld16;
-    for (int64_t j = threadIdx.x; j < N; j += blockDim.x) {
+    const int64_t nv = has1 ? N >> 2 : 0;
+    for (int64_t v = threadIdx.x; v < nv; v += blockDim.x) {
+      const int4 x = reinterpret_cast<const int4 *>(r0)[v], y = reinterpret_cast<const int4 *>(r1)[v];
+      reinterpret_cast<int4 *>(o)[v] =
+          make_int4((cap16(y.x, inf) << 16) | cap16(x.x, inf), (cap16(y.y, inf) << 16) | cap16(x.y, inf),
+                    (cap16(y.z, inf) << 16) | cap16(x.z, inf), (cap16(y.w, inf) << 16) | cap16(x.w, inf));
+    }
+    for (int64_t j = 4 * nv + threadIdx.x; j < N; j += blockDim.x) {
       const int lo = cap16(r0[j], inf), hi = has1 ? cap16(r1[j], inf) : kCap16;
       o[j] = (hi << 16) | lo;
     }
