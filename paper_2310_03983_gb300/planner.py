@@ -34,7 +34,7 @@ from . import (apsp_close_cta, apsp_fw, apsp_mlp_adam, apsp_mlp_backward, apsp_m
 CANDIDATES = (("fw", 0), ("rkleene", 128), ("rkleene", 256), ("rkleene", 512), ("rkleene", 1024), ("rkleene", 4096),
               ("cta", 0), ("squaring", 0))
 CTA_MAX_N = 1024  # beyond this one SM is far too slow to be worth timing
-IN_DIM = 12
+IN_DIM = 13
 FW16_MIN_N = 4096  # apsp_fw runs phase 3 on packed 16-bit pairs for int32 graphs this large
 HIDDEN = 64
 SMS = 152  # streaming multiprocessors of the GB300 the timing log was recorded on
@@ -69,6 +69,16 @@ def full_product_waves(n: int) -> int:
     return -(-t * t // SMS)
 
 
+def squaring_rounds(n: int) -> float:
+    """Time of one n x n product on 64 x 64 tiles, in units of half the time an SM takes for a pair of
+    them (gemm64.cu's own estimate): one or two tiles per SM at a time, whichever ends sooner."""
+    items = (-(-max(n, 1) // 64)) ** 2
+    left = items % (2 * SMS)
+    one = 1.27 * -(-items // SMS)
+    two = 2.0 * (items // (2 * SMS)) + (1.27 + 0.83 * min(left, SMS) / SMS if left else 0.0)
+    return one if items <= SMS else min(one, two)
+
+
 def features(n: int, density: float, dtype: str, algo: str, param: int) -> list[float]:
     """Feature vector of a (graph, configuration) pair, each entry scaled to about [0, 1]."""
     rk = algo == "rkleene"
@@ -80,7 +90,8 @@ def features(n: int, density: float, dtype: str, algo: str, param: int) -> list[
             1.0 if sq else 0.0,
             1.0 if algo == "fw" and dtype == "int32" and n >= FW16_MIN_N else 0.0,
             min(squaring_products(n, density, dtype), 15.0) / 15.0 if sq else 0.0,
-            math.log2(full_product_waves(n)) / 8.0]
+            math.log2(full_product_waves(n)) / 8.0,
+            math.log2(squaring_products(n, density, dtype) * squaring_rounds(n) * max(n, 1)) / 20.0 if sq else 0.0]
 
 
 def applicable(n: int):
