@@ -268,9 +268,6 @@ template <bool G>
 __global__ void __launch_bounds__(kFThreads, 1)
     fine_fw_kernel(const __grid_constant__ FineArgs a, const __grid_constant__ FineGraphs gs,
                    const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB) {
-  pdl_wait();
-  pdl_trigger();
-  if (a.run_if && !*a.run_if) return;
   extern __shared__ uint8_t smem_raw[];
   int *const smem0 = reinterpret_cast<int *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int wg = threadIdx.x / kFGroup, lane = threadIdx.x & 31;
@@ -297,14 +294,19 @@ __global__ void __launch_bounds__(kFThreads, 1)
     closing[g] = INT_MAX;
     fence_barrier_init();
   }
+  if (threadIdx.x == 0) {
+    tma_prefetch_desc(&mA);
+    tma_prefetch_desc(&mB);
+  }
   __syncthreads();
+  pdl_wait();  // after the set-up, before any global memory access
+  pdl_trigger();
+  if (a.run_if && !*a.run_if) return;
 
   if (wg == kFGroups) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kProducerRegs));
     if (lane != 0 || g >= a.groups) return;
     if ((threadIdx.x >> 5) % 4 < 2) {  // ------------------------- loads -------------------------
-      tma_prefetch_desc(&mA);
-      tma_prefetch_desc(&mB);
       uint32_t issued = 0, pars = 0;
       int s = a.s0, base = 0, before = 0;  // current stage, its first ticket, the items of the one before it
       StageCounts sc = launch_counts<G>(a, gs, s);

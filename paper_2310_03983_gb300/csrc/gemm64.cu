@@ -70,12 +70,6 @@ __device__ __forceinline__ int stages32(const int *words, int stages) {
 template <int KIND, bool P16>
 __global__ void __launch_bounds__(kFThreads, 1) gemm64_kernel(const __grid_constant__ G64Args a,
                                                               const __grid_constant__ G64Maps maps) {
-  pdl_wait();
-  pdl_trigger();
-  if ((a.skip && *a.skip) || (a.run_if && !*a.run_if)) return;
-  if (KIND == kSquare16 && !mode16(a.words)) return;
-  const int stages = KIND == kSquare32 ? stages32(a.words, a.stages) : a.stages;
-  if (stages <= 0) return;
   extern __shared__ uint8_t smem_raw[];
   int *const smem0 = reinterpret_cast<int *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int wg = threadIdx.x / kFGroup, lane = threadIdx.x & 31;
@@ -101,6 +95,12 @@ __global__ void __launch_bounds__(kFThreads, 1) gemm64_kernel(const __grid_const
     fence_barrier_init();
   }
   __syncthreads();
+  pdl_wait();  // after the set-up, before any global memory access
+  pdl_trigger();
+  if ((a.skip && *a.skip) || (a.run_if && !*a.run_if)) return;
+  if (KIND == kSquare16 && !mode16(a.words)) return;
+  const int stages = KIND == kSquare32 ? stages32(a.words, a.stages) : a.stages;
+  if (stages <= 0) return;
 
   if (wg == kFGroups) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kProducerRegs));

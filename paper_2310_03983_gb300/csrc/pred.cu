@@ -488,7 +488,8 @@ extern "C" int apsp_predecessors(const void *d, int64_t ldd, const void *w, int6
       p.wmax = words + kWBoundA;  // exact fp32 path when boundA + boundB < 2^24
       p.wmult = 1;
       p.skip = words + kWSkip;
-      r = launch_tgemm(kModeGemm, false, APSP_I32, mA, mB, mC, p, s);
+      r = gemm64_pays(n, n, n) ? launch_gemm64(false, APSP_I32, De, lde, We, lde, p, s)
+                               : launch_tgemm(kModeGemm, false, APSP_I32, mA, mB, mC, p, s);
     }
   }
   if (!r) {
