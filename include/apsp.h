@@ -106,7 +106,9 @@ int apsp_normalise(void *d, int64_t n, int64_t ld, int dtype, const void *inf, v
  * >= 0 or +infinity (float32); apsp_normalise produces that form.  C must not overlap A
  * or B (APSP_ERR_ARG).  K = 0 gives C = inf (or leaves C unchanged when accumulating);
  * M = 0 or N = 0 is a no-op.  When every base is 16-byte aligned and every leading
- * dimension a multiple of 4, the TMA-fed engine runs; otherwise a plain-load kernel.
+ * dimension a multiple of 4, the TMA-fed tiles run.  Otherwise, with ws == NULL, outside stream
+ * capture and from 2^24 (float32) or 2^26 (int32) pairs, they run on aligned copies in the
+ * library's pool; else a plain-load kernel.
  * int32 arithmetic is chosen on the device from the largest finite entries of A and B (a
  * scan): when they sum below 0x3FFF and the workspace has room for packed copies, the operands
  * are packed into 16-bit pairs and each DPX operation performs two (min,+) pairs; else, below
@@ -126,6 +128,7 @@ int tropical_gemm(void *C, const void *A, const void *B, int64_t M, int64_t N, i
  * by a (min,+) product with the closed tile; phase 3 updates every other tile by
  * D[i][j] = min(D[i][j], D[i][kb] (x) D[kb][j]).
  * tile: block size b; 0 selects the default (128).  Supported: 128.
+ * Matrices of 129..3200 vertices run the same phases over 64-vertex blocks (same workspace).
  * d must be 16-byte aligned.  The workspace holds 256 bytes of bound words (int32 matrices
  * whose (n - 1) * largest finite weight < 2^24 run in exact fp32 arithmetic on their bit
  * patterns; others in int32), when ld is not a multiple of 4 an aligned copy of the matrix
@@ -194,8 +197,10 @@ int apsp_fw_signed(void *d, int64_t n, int64_t ld, int dtype, const void *inf, v
  * the shortest paths of at most 2^max_iters edges.  Runs a1 first.  Costs n^3 (min,+) pairs per
  * product: O(n^3 log n) in the worst case against Floyd-Warshall's n^3, but only a few products
  * for graphs of small diameter.  d must be 16-byte aligned.  The workspace holds the 256 bytes
- * of bound words, the product matrix (n x round_up(n, 4) elements) and, when ld is not a
- * multiple of 4, an aligned copy of d.  int32 results equal apsp_fw's exactly; float32 results
+ * of bound words, the product matrix (n x round_up(n, 4) elements), when ld is not a
+ * multiple of 4 an aligned copy of d, and last, for int32 up to n = 4096, room for two sets of the
+ * matrix packed into 16-bit pairs (optional: a workspace without it is accepted).  With that room
+ * the products run on 16-bit pairs while the entries stay below half the cap of 0x3FFF.  int32 results equal apsp_fw's exactly; float32 results
  * differ from them only in summation order. */
 size_t apsp_squaring_workspace_bytes(int64_t n, int64_t ld, int dtype);
 int apsp_squaring(void *d, int64_t n, int64_t ld, int dtype, const void *inf, int max_iters,
@@ -248,7 +253,9 @@ size_t apsp_batched_workspace_bytes(int64_t count);
  * vertices are copied into a staging matrix in the workspace, each padded to whole 128-vertex
  * tiles; per 128-vertex block, one launch per phase runs it for every such graph (phase 3 on
  * packed 16-bit pairs, certified per graph as in apsp_fw, with an int32 pass for the graphs
- * whose certificate fails).  Every other graph goes to the persistent kernel.  Returns
+ * whose certificate fails).  When a step of all staged graphs together is at most 12 tiles of 64 x 64
+ * per SM, they are closed in 32 bits over 64-vertex blocks instead.  Every other graph goes to the
+ * persistent kernel.  Returns
  * apsp_batched_workspace_bytes(count) when no graph qualifies or dtype is APSP_F32.  The
  * staged path runs only when apsp_batched gets ns_host, a caller workspace of at least this
  * size and a sentinel above 0x3FFF; a staged graph whose device size, leading dimension or

@@ -10,6 +10,7 @@
 //   phase 3  D[i][j] = min(D[i][j], D[i][kb] (x) D[kb][j])      (i, j != kb)
 //            -- the rank-128 (min,+) update that carries essentially all n^3 of the work.
 // Phases 2 and 3 run on the TMA-fed tropical GEMM engine (tgemm.cu); phase 1 is one CTA.
+// Matrices of kFineMinN < n <= kFineMaxN vertices run the same phases over 64-vertex blocks (fine.cu).
 #include <algorithm>
 
 #include "closure.cuh"

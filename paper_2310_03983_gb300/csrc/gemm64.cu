@@ -239,7 +239,9 @@ __global__ void __launch_bounds__(kFThreads, 1) gemm64_kernel(const __grid_const
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           const bool in = ri + tm + 16 * i < a.M && cj + 4 * tn + 32 * (j >> 2) + (j & 3) < a.N;
-          if (KIND == kProduct) v[i][j] = min(v[i][j], o[i][j]);  // non-negative: fp32 orders as its bits
+          if (KIND == kProduct)
+            v[i][j] = a.is_float ? __float_as_int(fminf(__int_as_float(v[i][j]), __int_as_float(o[i][j])))
+                                 : min(v[i][j], o[i][j]);
           else diff |= in && v[i][j] != o[i][j];
         }
       __syncwarp();
