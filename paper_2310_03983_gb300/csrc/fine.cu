@@ -9,7 +9,7 @@
 // 64-vertex blocks cut the work of a link by eight (262 K pairs) and spread a panel or a matrix over
 // four times as many SMs.
 //
-// One launch runs one or two stages.  Stage s (of S = ceil(n / 64)) is
+// One launch runs one or two stages (a batch: up to eight).  Stage s (of S = ceil(n / 64)) is
 //   A(s): D[i][j] = min(D[i][j], D[i][s-1] (x) D[s-1][j]) for every tile outside block row / column
 //         s - 1 (phase 3 of block s - 1); tile (s, s) is then closed by Eq. 1 in registers (phase 1
 //         of block s); A(0) is only that closure;

@@ -27,6 +27,9 @@
 // weights; that pass's launches return at once when no graph needs it.  Results are identical
 // to closing each graph alone.
 //
+// A batch whose lockstep steps would leave most SMs idle (kFineBatchTilesPerSm) is staged the same way
+// and closed in 32 bits on 64-vertex blocks (fine.cu) instead of both passes.
+//
 // Float32 batches stage the same way (the sentinel and the padding are +infinity) and run only
 // the second pass, in fp32 (the engine's packed pair add and 3-input min), with no certificate.
 //
@@ -55,11 +58,11 @@ constexpr int kWBound = 8, kWRerun = 10;
 constexpr int kWFine = 16;  // [16..]: the counters of the 64-vertex-block closure (fine.cu)
 static_assert(kWFine + kFineWords <= 64, "word block");
 // A batch whose staged graphs have at most this many 64 x 64 tiles per SM in a step is closed with
-// 64-vertex blocks in 32 bits: its lockstep steps are bound by the chain of dependent tiles.
-#ifndef APSP_FBT
-#define APSP_FBT 12
-#endif
-constexpr int64_t kFineBatchTilesPerSm = APSP_FBT;
+// 64-vertex blocks in 32 bits: its lockstep steps are bound by the chain of dependent tiles.  Measured on
+// whole calls (int32, 64..1024 vertices; tiles per SM, 128-vertex lockstep / 64-vertex blocks): 2.3 591 /
+// 314 us, 5.2 799 / 604, 9.3 958 / 823, 23.3 1343 / 1419, 40.4 1726 / 1961 (float32 1417 / 1415 and
+// 1963 / 1949: even from 23 on).
+constexpr int64_t kFineBatchTilesPerSm = 12;
 constexpr int kPlanChunk = 4096;
 
 struct GroupSet {

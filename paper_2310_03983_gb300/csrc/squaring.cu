@@ -8,7 +8,8 @@
 // back into D and clears the iteration's "unchanged" word when any did.  The next product and
 // commit read that word on the device and return at once when it is still set, so the whole
 // loop is enqueued up front without a host round trip per iteration (and can be captured in
-// a CUDA graph), yet stops doing work at convergence.
+// a CUDA graph), yet stops doing work at convergence.  Up to kSquaring64MaxN vertices the loop is one
+// launch instead (gemm64.cu).
 #include <algorithm>
 
 #include "closure.cuh"
