@@ -199,9 +199,12 @@ int apsp_fw_signed(void *d, int64_t n, int64_t ld, int dtype, const void *inf, v
  * for graphs of small diameter.  d must be 16-byte aligned.  The workspace holds the 256 bytes
  * of bound words, the product matrix (n x round_up(n, 4) elements), when ld is not a
  * multiple of 4 an aligned copy of d, and last, for int32 up to n = 4096, room for two sets of the
- * matrix packed into 16-bit pairs (optional: a workspace without it is accepted).  With that room
- * the products run on 16-bit pairs while the entries stay below half the cap of 0x3FFF.  int32 results equal apsp_fw's exactly; float32 results
- * differ from them only in summation order. */
+ * matrix packed into 16-bit pairs (optional: a workspace without it is accepted, and then every
+ * product runs in 32 bits).  With that room the products run on 16-bit pairs while the entries
+ * stay below half the cap of 0x3FFF (checked on the device before each product, so no entry is ever
+ * cut short).  The other products run in one launch on 64 x 64 tiles or, where 128 x 128 ones are
+ * faster, in two launches each.  int32 results equal apsp_fw's exactly; float32 results differ from
+ * them only in summation order. */
 size_t apsp_squaring_workspace_bytes(int64_t n, int64_t ld, int dtype);
 int apsp_squaring(void *d, int64_t n, int64_t ld, int dtype, const void *inf, int max_iters,
                   void *ws, size_t ws_bytes, void *stream);

@@ -11,7 +11,7 @@
 // stage that changes nothing.  An item waits only for smaller tickets, held by running CTAs, so every
 // wait ends.  int32 matrices whose entries stay below half the 16-bit cap run on packed 16-bit
 // pairs, both packed forms of a product written by the tiles that compute it; when entries outgrow
-// that, the remaining products run on 32 bits.
+// that, the remaining products run on 32 bits (here, or on 128 x 128 tiles in squaring.cu's loop).
 #include <algorithm>
 #include <atomic>
 
@@ -27,10 +27,14 @@ constexpr int kSPacked = 2;     // the packed forms exist (square_prep_kernel ra
 constexpr int kSAbort = 3;      // 1 + the stage at which they stopped (0: they finished)
 constexpr int kSCtr16 = 4;      // ticket, unused, done (16-bit stages)
 constexpr int kSCtr32 = 8;      // the same for the 32-bit stages
+constexpr int kSMaxStages = 12; // products that close kSquaring64MaxN vertices
 constexpr int kSChanged16 = 12; // per stage: something changed
-constexpr int kSMax16 = 28;     // per stage: largest finite entry written
-constexpr int kSChanged32 = 44;
-constexpr int kSMaxStages = 16;
+constexpr int kSMax16 = 24;     // per stage: largest finite entry written
+constexpr int kSChanged32 = 36;
+static_assert(int64_t(1) << kSMaxStages >= kSquaring64MaxN - 1, "stages");
+static_assert(kSChanged16 + kSMaxStages <= kSMax16 && kSMax16 + kSMaxStages <= kSChanged32 &&
+                  kSChanged32 + kSMaxStages <= kSquareUnchanged && kSquareUnchanged + kSMaxStages <= kSquareSkip &&
+                  kSquareSkip < 64, "squaring words");
 
 enum { kProduct = 0, kSquare32 = 1, kSquare16 = 2, kArgChunk = 3 };
 
@@ -384,13 +388,19 @@ __global__ void __launch_bounds__(256) square_prep_kernel(int *d, int64_t ld, in
 }
 
 // The last complete set of the 16-bit stages back into the int32 matrix (a set that no stage changed
-// equals the one before it).  A word is two columns; rows are 16-byte aligned.
+// equals the one before it).  A word is two columns; rows are 16-byte aligned.  Also sets the words by
+// which a loop of one launch per product (squaring.cu) skips what is done: words[kSquareSkip] for its
+// first product, words[kSquareUnchanged + t] ("product t changed nothing") for product t + 1.
 __global__ void __launch_bounds__(256) square_unpack_kernel(int *d, int64_t ld, int n, const int *A0, const int *A1,
-                                                            int64_t lda16, int stages, int inf, const int *words) {
+                                                            int64_t lda16, int stages, int inf, int *words) {
   pdl_wait();
   pdl_trigger();
-  if (!mode16(words)) return;
-  const int done = words[kSAbort] ? words[kSAbort] - 1 : stages;
+  const bool packed = mode16(words);
+  const int done = !packed ? 0 : words[kSAbort] ? words[kSAbort] - 1 : stages;
+  if (blockIdx.x == 0 && threadIdx.x < kSMaxStages)
+    words[kSquareUnchanged + threadIdx.x] = done == stages || (int)threadIdx.x != done - 1;
+  if (blockIdx.x == 0 && threadIdx.x == 0) words[kSquareSkip] = done > 0;
+  if (!packed) return;
   const int *A = done & 1 ? A1 : A0;
   for (int i = blockIdx.x; i < n; i += gridDim.x)
     for (int j = 4 * threadIdx.x; j < n; j += 4 * blockDim.x) {
@@ -437,16 +447,16 @@ int groups_for(int64_t items) { return items <= sm_count() || one_group(items) <
 
 }  // namespace
 
-// Rounds of 128 x 128 tiles (four units of work each, one per SM) against rounds of 64 x 64 tiles, which
-// must win by 15% on paper: at the edge they lose (1000 x 1300 x 700 int32, 82 us against 77;
-// 2000^3 in 32 bits, 513 against 490), inside it they gain (1024^3 fp32 67 against 121 us, 512^3 22
-// against 62, 300 x 300 x 6000 205 against 670, 4000 x 1300 x 64 26 against 29).
-bool gemm64_pays(int64_t M, int64_t N, int64_t K) {
+// Rounds of 128 x 128 tiles (four units of work each, one per SM) against rounds of 64 x 64 tiles.  A
+// product on its own must win by 15% on paper (percent = 85): at the edge they lose (1000 x 1300 x 700
+// int32, 82 us against 77; 2000^3 in 32 bits, 513 against 490), inside it they gain (1024^3 fp32 67 against
+// 121 us, 512^3 22 against 62, 300 x 300 x 6000 205 against 670, 4000 x 1300 x 64 26 against 29).
+bool gemm64_pays(int64_t M, int64_t N, int64_t K, int percent) {
   if (K <= 0 || M > INT32_MAX / 2 || N > INT32_MAX / 2) return false;
   const int64_t t128 = cdiv(M, kBM) * cdiv(N, kBN), t64 = cdiv(M, kFB) * cdiv(N, kFB);
   if (t64 > INT32_MAX / 2) return false;
   const int64_t c64 = groups_for(t64) == 1 ? one_group(t64) : two_groups(t64);
-  return 100 * c64 < 85 * 400 * cdiv(t128, sm_count());
+  return 100 * c64 < percent * 400 * cdiv(t128, sm_count());
 }
 
 int launch_gemm64(bool acc, int dtype, const void *A, int64_t lda, const void *B, int64_t ldb, const TileProblem &p,
@@ -503,50 +513,56 @@ size_t squaring64_bytes(int64_t n, int dtype) {
   return 2 * ((size_t)round_up(n * sq_lda16(n) * 4, 256) + (size_t)round_up(((n + 1) >> 1) * sq_ldb16(n) * 4, 256));
 }
 
-int squaring64(void *d, int64_t n, int64_t ld, int dtype, int inf_i, float inf_f, int iters, int *words, int *C, int64_t ldc,
-               void *packed, cudaStream_t s) {
-  static_assert(kSChanged32 + kSMaxStages <= 64 && kSMax16 + kSMaxStages <= kSChanged32 &&
-                    kSChanged16 + kSMaxStages <= kSMax16, "squaring words");
-  if (iters > kSMaxStages) return APSP_ERR_ARG;
-  const bool isf = dtype == APSP_F32;
-  int r;
+static G64Args square_args(int64_t n, int iters, int *words) {
   G64Args a = {};
-  G64Maps m = {};
   a.M = a.N = a.K = (int)n;
   a.tiles_n = (int)cdiv(n, kFB);
   a.items = a.tiles_n * a.tiles_n;
   a.stages = iters;
   a.groups = groups_for(a.items);
-  a.is_float = isf;
-  a.inf = isf ? 0x7f800000 : inf_i;
   a.words = words;
   a.status = status_word();
+  return a;
+}
+
+int squaring64_packed(void *d, int64_t n, int64_t ld, int inf_i, int iters, int *words, void *packed, cudaStream_t s) {
+  if (iters > kSMaxStages) return APSP_ERR_ARG;
+  int r;
+  G64Args q = square_args(n, iters, words);
+  G64Maps mq = {};
+  q.inf = inf_i;
+  q.K = (int)((n + 1) >> 1);
+  q.lda16 = sq_lda16(n);
+  q.ldb16 = sq_ldb16(n);
+  uint8_t *at = reinterpret_cast<uint8_t *>(packed);
+  for (int k = 0; k < 2; ++k) {
+    q.pa[k] = reinterpret_cast<int *>(at);
+    at += round_up(n * q.lda16 * 4, 256);
+    q.pb[k] = reinterpret_cast<int *>(at);
+    at += round_up((int64_t)q.K * q.ldb16 * 4, 256);
+    if ((r = maps64(&mq.A[k], &mq.B[k], q.pa[k], n, q.K, q.lda16, q.pb[k], n, q.ldb16, APSP_I32))) return r;
+  }
   const int grid = (int)std::min<int64_t>(n, (int64_t)sm_count() * 4);
   int *D = reinterpret_cast<int *>(d);
-  if (!isf && packed && inf_i > kCap16) {  // a1 and the 16-bit stages
-    G64Args q = a;
-    G64Maps mq = {};
-    q.K = (int)((n + 1) >> 1);
-    q.lda16 = sq_lda16(n);
-    q.ldb16 = sq_ldb16(n);
-    uint8_t *at = reinterpret_cast<uint8_t *>(packed);
-    for (int k = 0; k < 2; ++k) {
-      q.pa[k] = reinterpret_cast<int *>(at);
-      at += round_up(n * q.lda16 * 4, 256);
-      q.pb[k] = reinterpret_cast<int *>(at);
-      at += round_up((int64_t)q.K * q.ldb16 * 4, 256);
-      if ((r = maps64(&mq.A[k], &mq.B[k], q.pa[k], n, q.K, q.lda16, q.pb[k], n, q.ldb16, APSP_I32))) return r;
-    }
-    launch_pdl(square_prep_kernel, grid, 256, 0, s, D, ld, (int)n, q.pa[0], q.lda16, q.pb[0], q.ldb16, inf_i, words,
-               status_word());
-    APSP_LAUNCH_CHECK();
-    if ((r = launch64<kSquare16, true>(q, mq, s))) return r;
-    launch_pdl(square_unpack_kernel, grid, 256, 0, s, D, ld, (int)n, q.pa[0], q.pa[1], q.lda16, iters, inf_i, words);
-    APSP_LAUNCH_CHECK();
-  } else if ((r = launch_normalise(d, n, ld, dtype, inf_i, inf_f, isf ? nullptr : words, s))) {
-    return r;
-  }
-  a.out[0] = D;
+  launch_pdl(square_prep_kernel, grid, 256, 0, s, D, ld, (int)n, q.pa[0], q.lda16, q.pb[0], q.ldb16, inf_i, words,
+             status_word());
+  APSP_LAUNCH_CHECK();
+  if ((r = launch64<kSquare16, true>(q, mq, s))) return r;
+  launch_pdl(square_unpack_kernel, grid, 256, 0, s, D, ld, (int)n, q.pa[0], q.pa[1], q.lda16, iters, inf_i, words);
+  APSP_LAUNCH_CHECK();
+  return APSP_OK;
+}
+
+int squaring64(void *d, int64_t n, int64_t ld, int dtype, int inf_i, int iters, int *words, int *C, int64_t ldc,
+               cudaStream_t s) {
+  if (iters > kSMaxStages) return APSP_ERR_ARG;
+  const bool isf = dtype == APSP_F32;
+  int r;
+  G64Args a = square_args(n, iters, words);
+  G64Maps m = {};
+  a.is_float = isf;
+  a.inf = isf ? 0x7f800000 : inf_i;
+  a.out[0] = reinterpret_cast<int *>(d);
   a.out[1] = C;
   a.ldo[0] = ld;
   a.ldo[1] = ldc;
@@ -555,7 +571,8 @@ int squaring64(void *d, int64_t n, int64_t ld, int dtype, int inf_i, float inf_f
   for (int k = 0; k < 2; ++k)
     if ((r = maps64(&m.A[k], &m.B[k], a.out[k], n, n, a.ldo[k], a.out[k], n, a.ldo[k], dtype))) return r;
   if ((r = launch64<kSquare32, false>(a, m, s))) return r;
-  launch_pdl(square_finish_kernel, grid, 256, 0, s, D, ld, (int)n, C, ldc, iters, words);
+  const int grid = (int)std::min<int64_t>(n, (int64_t)sm_count() * 4);
+  launch_pdl(square_finish_kernel, grid, 256, 0, s, a.out[0], ld, (int)n, C, ldc, iters, words);
   APSP_LAUNCH_CHECK();
   return APSP_OK;
 }

@@ -8,8 +8,9 @@
 // back into D and clears the iteration's "unchanged" word when any did.  The next product and
 // commit read that word on the device and return at once when it is still set, so the whole
 // loop is enqueued up front without a host round trip per iteration (and can be captured in
-// a CUDA graph), yet stops doing work at convergence.  Up to kSquaring64MaxN vertices the loop is one
-// launch instead (gemm64.cu).
+// a CUDA graph), yet stops doing work at convergence.  Matrices whose products are faster on 64 x 64
+// tiles run the whole loop in one launch instead, and int32 ones up to kSquaring64MaxN vertices start
+// with the products that fit packed 16-bit pairs, also in one launch (gemm64.cu).
 #include <algorithm>
 
 #include "closure.cuh"
@@ -24,6 +25,8 @@ constexpr int kMaxIters = 48;       // 8 + 48 words fit in the 256-byte bound-wo
 
 __global__ void __launch_bounds__(256) commit_kernel(int *D, int64_t ldd, const int *C, int64_t ldc, int64_t n,
                                                      const int *skip, int *unchanged) {
+  pdl_wait();
+  pdl_trigger();
   if (skip && *skip) return;
   bool changed = false;
   for (int64_t i = blockIdx.x; i < n; i += gridDim.x) {
@@ -48,9 +51,6 @@ int iters_for(int64_t n) {
 
 }  // namespace
 
-}  // namespace apsp
-
-namespace apsp {
 // What a call cannot do without; the packed operands of small int32 matrices (last) are optional.
 static size_t squaring_required_bytes(int64_t n, int64_t ld) {
   const size_t mat = (size_t)round_up(n * round_up(n, 4) * 4, 256);
@@ -88,16 +88,19 @@ extern "C" int apsp_squaring(void *d, int64_t n, int64_t ld, int dtype, const vo
     ws_bytes = need;
   }
   void *packed = need > base && ws_bytes >= need ? reinterpret_cast<uint8_t *>(ws) + base : nullptr;
-  const bool small = n <= kSquaring64MaxN;
+  // No more products than can change anything; 16-bit ones first, then the 32-bit ones.
+  const int needed = std::min(iters, iters_for(n));
+  const bool packed16 = packed && needed > 0 && inf_i > kCap16, tiles64 = squaring64_pays(n, packed16);
   int r = APSP_OK;
   uint8_t *wsp = reinterpret_cast<uint8_t *>(ws);
-  int *words = reinterpret_cast<int *>(wsp);  // [0]: largest finite weight, [1]: 0, [8 + t]: unchanged flags
+  int *words = reinterpret_cast<int *>(wsp);  // [0]: largest finite weight, [1]: 0, then the flags
+  int *unchanged = words + (packed16 ? kSquareUnchanged : kWordsUnchanged);
   wsp += kFlagBytes;
   const int64_t lde = round_up(n, 4);
   int *C = reinterpret_cast<int *>(wsp);
   wsp += round_up(n * lde * 4, 256);
-  if (cudaMemsetAsync(words, 0, small ? kFlagBytes : 16, s) != cudaSuccess) r = APSP_ERR_CUDA;
-  if (!r && !small && cudaMemsetAsync(words + kWordsUnchanged, 1, 4 * kMaxIters, s) != cudaSuccess) r = APSP_ERR_CUDA;
+  if (cudaMemsetAsync(words, 0, kFlagBytes, s) != cudaSuccess) r = APSP_ERR_CUDA;
+  if (!r && !packed16 && !tiles64 && cudaMemsetAsync(unchanged, 1, 4 * kMaxIters, s) != cudaSuccess) r = APSP_ERR_CUDA;
   void *work = d;
   int64_t ldw = ld;
   if (!r && ld % 4 != 0) {  // the engine needs 16-byte rows: work on an aligned copy
@@ -105,20 +108,16 @@ extern "C" int apsp_squaring(void *d, int64_t n, int64_t ld, int dtype, const vo
     work = wsp;
     r = launch_copy2d(work, ldw, d, ld, n, n, s);
   }
-  // Small matrices: the whole loop in one launch on 64 x 64 tiles (gemm64.cu), no more products than
-  // can change anything.
-  const int needed = std::min(iters, iters_for(n));
-  if (!r && small && needed > 0) {
-    r = squaring64(work, n, ldw, dtype, inf_i, inf_f, needed, words, C, lde, packed, s);
-  } else if (!r) {
-    r = launch_normalise(work, n, ldw, dtype, inf_i, inf_f, dtype == APSP_I32 ? words : nullptr, s);
-  }
+  if (!r) r = packed16 ? squaring64_packed(work, n, ldw, inf_i, needed, words, packed, s)
+                       : launch_normalise(work, n, ldw, dtype, inf_i, inf_f, dtype == APSP_I32 ? words : nullptr, s);
+  if (!r && tiles64 && needed > 0) r = squaring64(work, n, ldw, dtype, inf_i, needed, words, C, lde, s);
+  const int loop = tiles64 ? 0 : needed;
   CUtensorMap mA, mB, mC;
-  if (!r) r = make_operand_maps(work, n, n, ldw, dtype, &mA, &mB, nullptr);
-  if (!r) r = make_operand_maps(C, n, n, lde, dtype, nullptr, nullptr, &mC);
+  if (!r && loop) r = make_operand_maps(work, n, n, ldw, dtype, &mA, &mB, nullptr);
+  if (!r && loop) r = make_operand_maps(C, n, n, lde, dtype, nullptr, nullptr, &mC);
   const int64_t cap = (int64_t)sm_count() * 8;
-  for (int t = 0; t < iters && !r && !small; ++t) {
-    const int *skip = t > 0 ? words + kWordsUnchanged + t - 1 : nullptr;
+  for (int t = 0; t < loop && !r; ++t) {
+    const int *skip = t > 0 ? unchanged + t - 1 : packed16 ? words + kSquareSkip : nullptr;
     TileProblem p = {};
     p.M = n; p.N = n; p.K = n;
     p.tiles_m = cdiv(n, kBM);
@@ -134,8 +133,8 @@ extern "C" int apsp_squaring(void *d, int64_t n, int64_t ld, int dtype, const vo
     p.skip = skip;
     r = launch_tgemm(kModeGemm, false, dtype, mA, mB, mC, p, s);
     if (!r) {
-      commit_kernel<<<(int)(n < cap ? n : cap), 256, 0, s>>>(reinterpret_cast<int *>(work), ldw, C, lde, n, skip,
-                                                             words + kWordsUnchanged + t);
+      launch_pdl(commit_kernel, (int)(n < cap ? n : cap), 256, 0, s, reinterpret_cast<int *>(work), ldw, C, lde, n, skip,
+                 unchanged + t);
       note_launch();
       if (cudaGetLastError() != cudaSuccess) r = APSP_ERR_CUDA;
     }
