@@ -340,14 +340,27 @@ __device__ __forceinline__ int *graph_base(const BatchArgs &a, int g, int &n, in
   return a.pool + off;
 }
 
+// About the time of a graph of n vertices on one CTA, and on a cluster of csize CTAs that share its panel
+// and remaining tiles, in units of 0.31 us: fitted to a graph's measured time in us, on one CTA n = 32 14, 64
+// 25, 100 36, 128 45, 129 122, 200 175, 256 215, on four 129 105, 200 143, 256 170.  The first terms close
+// the b diagonal tiles, the last is its panel and remaining tiles.
+__device__ __forceinline__ float lone_cost(int n) {
+  const float m = (float)n, b = (float)(((unsigned)n + kSlabM - 1) / kSlabM);
+  return 1.04f * m + 12.0f * b + (b * b - 1.0f) * (21.0f + 0.444f * m);
+}
+__device__ __forceinline__ float cluster_cost(int n, int csize) {
+  const float m = (float)n, b = (float)(((unsigned)n + kSlabM - 1) / kSlabM), c = (float)csize;
+  return 1.04f * m + 12.0f * b + (ceilf(2.0f * (b - 1.0f) / c) + ceilf((b - 1.0f) * (b - 1.0f) / c)) * (51.0f + 0.303f * m);
+}
+
 // The persistent kernel runs as clusters of csize CTAs (csize = 1 without clusters), in two
 // stages.  Stage 1: the leading run of the queue order whose graphs are each too large for
-// one CTA to close within the batch's average time per CTA (the order is largest first), or all
-// graphs above one tile when there is a cluster for each, is closed one graph at a time by whole clusters: rank 0 takes the next
-// entry and writes it into every CTA's shared memory through distributed shared memory, and
-// hardware cluster barriers separate the steps.  Stage 2: every CTA pulls the remaining
-// graphs from its own counter and closes each alone, with no cluster barrier at all.  No CTA
-// ever spins.
+// one CTA to close within the batch's average time per CTA (the order is largest first), or those
+// above one tile when clusters close them sooner, is closed one graph at a time by whole
+// clusters: rank 0 takes the next entry and writes it into every CTA's shared memory through
+// distributed shared memory, and hardware cluster barriers separate the steps.  Stage 2: every CTA
+// pulls the remaining graphs from its own counter and closes each alone, with no cluster barrier at
+// all.  No CTA ever spins.
 template <typename S>
 __global__ void __launch_bounds__(kBThreads, 1) batched_kernel(const BatchArgs a) {
   extern __shared__ uint8_t smem_raw[];
@@ -372,24 +385,41 @@ __global__ void __launch_bounds__(kBThreads, 1) batched_kernel(const BatchArgs a
   int nbig = 0;
   if (csize > 1) {
     __shared__ double s_work[kBThreads / 32];
+    __shared__ float s_lone[kBThreads / 32], s_move[kBThreads / 32];
+    __shared__ int s_small[kBThreads / 32], s_big;  // largest graph of one tile; largest that would move to a cluster
     double w = 0.0;
+    float lone = 0.0f;
+    int small = 0, first = 0;  // first: vertices of this thread's first entry
     for (int k = threadIdx.x; k < a.nq; k += kBThreads) {
       const int g = a.order ? a.order[k] : k;
       if (g >= 0 && g < a.count) {
-        const double n = (double)max(a.ns[g], 0);
+        const int v = max(a.ns[g], 0);
+        const double n = (double)v;
         w += n * n * n;
+        if (v > 0) lone += lone_cost(v);
+        if (v <= kSlabM) small = max(small, v);
+        if (k == (int)threadIdx.x) first = v;
       }
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-    if ((threadIdx.x & 31) == 0) s_work[threadIdx.x >> 5] = w;
-    if (threadIdx.x == 0) s_nbig = s_ntile = (int)a.nq;
+    for (int o = 16; o > 0; o >>= 1) {
+      w += __shfl_xor_sync(0xffffffffu, w, o);
+      lone += __shfl_xor_sync(0xffffffffu, lone, o);
+    }
+    small = __reduce_max_sync(0xffffffffu, small);
+    if ((threadIdx.x & 31) == 0) {
+      s_work[threadIdx.x >> 5] = w;
+      s_lone[threadIdx.x >> 5] = lone;
+      s_small[threadIdx.x >> 5] = small;
+    }
+    if (threadIdx.x == 0) {
+      s_nbig = s_ntile = (int)a.nq;
+      s_big = 0;
+    }
     __syncthreads();
     double total = 0.0;
 #pragma unroll
     for (int i = 0; i < kBThreads / 32; ++i) total += s_work[i];
-    // ... or, when the graphs above one tile are no more than the clusters, all of those: a cluster
-    // shares their panel and remaining tiles (n = 256 on one CTA: six 128^3 products in turn).
     const double big3 = fmax(0.5 * total / (double)gridDim.x, (double)(64 * csize) * (64 * csize) * (64 * csize));
     int first_small = (int)a.nq, first_tile = (int)a.nq;
     for (int k = threadIdx.x; k < a.nq; k += kBThreads) {
@@ -405,7 +435,34 @@ __global__ void __launch_bounds__(kBThreads, 1) batched_kernel(const BatchArgs a
     atomicMin(&s_ntile, first_tile);
     __syncthreads();
     nbig = s_nbig;
-    if (s_ntile <= (int)gridDim.x / csize) nbig = max(nbig, s_ntile);
+    // ... and the others above one tile, when there is a cluster for each and the batch ends sooner that
+    // way.  Left alone, the largest of them takes lone_cost on one CTA while the other CTAs close the
+    // graphs of one tile; on clusters, every CTA has its share of both (the last of which ends half
+    // a graph late on average).  Measured (int32, us, on clusters / alone; share of the line below): 16 graphs of
+    // 256 beside 400 of 64 190 / 235 (0.69), 19 beside 1000 of 32 207 / 237 (0.90), 16 of 200 beside 400 of 128
+    // 229 / 196 (1.23), 19 of 256 beside 1000 of 100 363 / 288 (1.76).
+    // Every CTA adds in the same order, so all come to the same choice.
+    const int ntile = s_ntile;
+    if (ntile > nbig && ntile <= min((int)gridDim.x / csize, kBThreads)) {
+      const bool in = (int)threadIdx.x < ntile && first > 0, moved = in && (int)threadIdx.x >= nbig;
+      float move = (moved ? (float)csize * cluster_cost(first, csize) : 0.0f) - (in ? lone_cost(first) : 0.0f);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) move += __shfl_xor_sync(0xffffffffu, move, o);
+      const int big = __reduce_max_sync(0xffffffffu, moved ? first : 0);
+      if ((threadIdx.x & 31) == 0) {
+        s_move[threadIdx.x >> 5] = move;
+        if (big > 0) atomicMax(&s_big, big);
+      }
+      __syncthreads();
+      float share = 0.0f;
+      small = 0;
+#pragma unroll
+      for (int i = 0; i < kBThreads / 32; ++i) {
+        share += s_lone[i] + s_move[i];
+        small = max(small, s_small[i]);
+      }
+      if (share <= (float)gridDim.x * (lone_cost(s_big) - 0.5f * lone_cost(small))) nbig = ntile;
+    }
     cl.sync();
   }
 
