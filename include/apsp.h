@@ -289,8 +289,11 @@ int apsp_batched(void *pool, const int64_t *offsets, const int32_t *ns, const in
  * float32: each sum rounded once (round to nearest), ties to the smallest k.  From n = 128 the
  * argmin runs on the (min,+) tiles: a product finds the 64-deep chunk of k that holds each minimum,
  * a second pass the index in it; the workspace then holds four n x round_up(n, 4) matrices (clean
- * copies of d, w and w transposed, and the chunks).  With a smaller workspace (256 bytes are
- * accepted), and without one while the stream is captured, a direct kernel runs instead. */
+ * copies of d, w and w transposed, and the chunks), but never more than about 1 GiB (n = 8192):
+ * beyond that it holds strips of them and the passes run strip by strip.  Without a workspace that
+ * scratch comes from the library's pool, which keeps it for later calls until
+ * apsp_workspace_pool_trim.  With a smaller workspace (256 bytes are accepted), and without one
+ * while the stream is captured, a direct kernel runs instead. */
 size_t apsp_predecessors_workspace_bytes(int64_t n, int dtype);
 int apsp_predecessors(const void *d, int64_t ldd, const void *w, int64_t ldw, int32_t *pred,
                       int64_t ldp, int64_t n, int dtype, const void *inf, void *ws,

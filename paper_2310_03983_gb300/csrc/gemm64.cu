@@ -489,12 +489,12 @@ int launch_gemm64(bool acc, int dtype, const void *A, int64_t lda, const void *B
   return r;
 }
 
-int launch_arg_chunks(const float *A, int64_t lda, const float *B, int64_t ldb, int64_t n, int *out, int64_t ldo,
-                      cudaStream_t s) {
+int launch_arg_chunks(const float *A, int64_t lda, const float *B, int64_t ldb, int64_t M, int64_t N, int64_t K, int *out,
+                      int64_t ldo, cudaStream_t s) {
   G64Args a = {};
-  a.M = a.N = a.K = (int)n;
-  a.tiles_n = (int)cdiv(n, kFB);
-  a.items = a.tiles_n * a.tiles_n;
+  a.M = (int)M; a.N = (int)N; a.K = (int)K;
+  a.tiles_n = (int)cdiv(N, kFB);
+  a.items = (int)(cdiv(M, kFB) * a.tiles_n);
   a.stages = 1;
   a.groups = groups_for(a.items);
   a.is_float = 1;
@@ -504,7 +504,7 @@ int launch_arg_chunks(const float *A, int64_t lda, const float *B, int64_t ldb, 
   a.status = status_word();
   G64Maps m = {};
   int r;
-  if ((r = maps64(&m.A[0], &m.B[0], A, n, n, lda, B, n, ldb, APSP_F32))) return r;
+  if ((r = maps64(&m.A[0], &m.B[0], A, M, K, lda, B, N, ldb, APSP_F32))) return r;
   return launch64<kArgChunk, false>(a, m, s);
 }
 

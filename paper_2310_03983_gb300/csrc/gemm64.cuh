@@ -14,11 +14,11 @@ bool gemm64_pays(int64_t M, int64_t N, int64_t K, int percent = 85);
 int launch_gemm64(bool acc, int dtype, const void *A, int64_t lda, const void *B, int64_t ldb, const TileProblem &p,
                   cudaStream_t s);
 
-// float32, aligned n x n operands: out[i][j] = the first chunk of kArgChunkLen consecutive k that holds
-// min_k A[i][k] + B[k][j], or -1 when that minimum is +infinity.
+// float32, aligned operands, M x K and K x N: out[i][j] = the first chunk of kArgChunkLen consecutive k that
+// holds min_k A[i][k] + B[k][j], or -1 when that minimum is +infinity.
 constexpr int kArgChunkLen = 64;
-int launch_arg_chunks(const float *A, int64_t lda, const float *B, int64_t ldb, int64_t n, int *out, int64_t ldo,
-                      cudaStream_t s);
+int launch_arg_chunks(const float *A, int64_t lda, const float *B, int64_t ldb, int64_t M, int64_t N, int64_t K, int *out,
+                      int64_t ldo, cudaStream_t s);
 
 // Repeated squaring, D <- D (x) D `iters` times or until nothing changes, up to kSquaring64MaxN vertices (the
 // stages wait on one another inside one launch).  D 16-byte aligned, ld % 4 == 0; words: the call's 64

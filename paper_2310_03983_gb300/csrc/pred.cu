@@ -18,6 +18,7 @@
 // argmin kernel (add, compare, two selects per (i, j, k)) computes pred instead.  float32
 // matrices cannot carry an index in their low bits (their sums round): above a few vertices a product
 // notes which chunk of k holds each minimum and a second pass finds the index in it (below).
+#include <algorithm>
 #include <climits>
 
 #include "closure.cuh"
@@ -301,39 +302,64 @@ __device__ __forceinline__ int64_t cdiv_dev(int64_t a, int64_t b) { return (a + 
 //      equals their minimum, both operands contiguous.
 // Measured (the direct kernel in brackets): n = 128 30 us (65), 512 46 (190), 1000 121 (320), 3000
 // 1948 (3716), 8192 31.9 ms (73.1).
+// The copies would grow with n^2 (16 n^2 bytes), so beyond kChunkedScratch the three steps run once per
+// pair of a strip of d's rows and a strip of w's columns, with room for one strip of each.
 constexpr int64_t kChunkedMinN = 128, kChunkedMaxN = 1 << 20;
-size_t chunked_bytes(int64_t n) { return 4 * enc_bytes(n); }
+constexpr size_t kChunkedScratch = size_t(1) << 30;
 
+// Scratch for strips of s rows of d and s columns of w: De and Wt (s rows of enc_ld(n)), We (n rows of
+// enc_ld(s)), the chunks (s rows of enc_ld(s)).
+size_t strip_bytes(int64_t rows, int64_t cols) { return (size_t)round_up(rows * enc_ld(cols) * 4, 256); }
+size_t chunked_bytes(int64_t n, int64_t s) { return 2 * strip_bytes(s, n) + strip_bytes(n, s) + strip_bytes(s, s); }
+
+// The strips' width: n, or about n / 2, n / 3, ... in whole tiles (s stays a multiple of 32, the cleaning
+// kernel's tile, and 16-byte rows), the first whose scratch fits.
+int64_t strip_edge(int64_t n) {
+  int64_t s = n;
+  for (int64_t t = 2; chunked_bytes(n, s) > kChunkedScratch && s > 64; ++t) s = round_up(cdiv(n, t), 64);
+  return s;
+}
+
+// Step 1 for rows i0 .. i0 + mi of d (into De) and columns j0 .. j0 + nj of w (into We and Wt; nj = 0: they
+// are there already), both on 32 x 32 tiles of the n x n matrices; i0 and j0 are multiples of 32.  STRIPS
+// false: the whole of both (the range checks cost 0.6% of a whole call at n = 3000).
+template <bool STRIPS>
 __global__ void __launch_bounds__(256) pred_clean_kernel(const float *d, int64_t ldd, const float *w, int64_t ldw, float *De,
-                                                         float *We, float *Wt, int64_t lde, int64_t n, float inf,
-                                                         unsigned int *st) {
+                                                         float *We, float *Wt, int64_t lde, int64_t lds, int64_t n, int64_t i0,
+                                                         int64_t mi, int64_t j0, int64_t nj, float inf, unsigned int *st) {
   __shared__ float tile[32][33];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const float big = __int_as_float(0x7f800000);
   bool bad = false;
-  const int64_t nt = cdiv_dev(n, 32);
-  for (int64_t t = blockIdx.x; t < nt * nt; t += gridDim.x) {
-    const int64_t i0 = t / nt * 32, j0 = (t - t / nt * nt) * 32, j = j0 + tx;
+  const int64_t nt = cdiv_dev(n, 32), first = !STRIPS || nj ? 0 : i0, rows = !STRIPS || nj ? nt : cdiv_dev(mi, 32);
+  if (!STRIPS) {
+    i0 = j0 = 0;
+    lds = lde;
+  }
+  for (int64_t t = blockIdx.x; t < rows * nt; t += gridDim.x) {
+    const int64_t ti = first + t / nt * 32, tj = (t - t / nt * nt) * 32, j = tj + tx;
+    const bool dpart = !STRIPS || (ti >= i0 && ti < i0 + mi), wpart = !STRIPS || (tj >= j0 && tj < j0 + nj);
+    if (!dpart && !wpart) continue;
     __syncthreads();
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const int64_t i = i0 + ty + 8 * u;
+      const int64_t i = ti + ty + 8 * u;
       float dv = big, wv = big;
       if (i < n && j < n) {
-        dv = PredOps<float>::fix(d[i * ldd + j], inf, bad);
-        if (i != j) wv = PredOps<float>::fix(w[i * ldw + j], inf, bad);
+        if (dpart) dv = PredOps<float>::fix(d[i * ldd + j], inf, bad);
+        if (wpart && i != j) wv = PredOps<float>::fix(w[i * ldw + j], inf, bad);
       }
       tile[ty + 8 * u][tx] = wv;
       if (i < n && j < lde) {  // columns n .. lde - 1 are +infinity
-        De[i * lde + j] = dv;
-        We[i * lde + j] = wv;
+        if (dpart) De[(i - i0) * lde + j] = dv;
+        if (wpart && j - j0 < lds) We[i * lds + j - j0] = wv;
       }
     }
     __syncthreads();
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const int64_t r = j0 + ty + 8 * u, c = i0 + tx;
-      if (r < n && c < lde) Wt[r * lde + c] = tile[tx][ty + 8 * u];
+      const int64_t r = tj + ty + 8 * u, c = ti + tx;
+      if (wpart && r < n && c < lde) Wt[(r - j0) * lde + c] = tile[tx][ty + 8 * u];
     }
   }
   if (__syncthreads_or(bad) && threadIdx.x == 0) flag_status(st, APSP_ERR_DOMAIN);
@@ -342,19 +368,26 @@ __global__ void __launch_bounds__(256) pred_clean_kernel(const float *d, int64_t
 // Step 3: a block takes 64 columns of kPickRows rows; four lanes per entry, 16 of its k each.
 constexpr int kPickRows = 16;
 
+template <bool STRIPS>
 __global__ void __launch_bounds__(256) pred_pick_kernel(const float *De, const float *Wt, const int *chunk, int64_t lde,
-                                                        int *pred, int64_t ldp, int64_t n) {
+                                                        int64_t lds, int *pred, int64_t ldp, int64_t i0, int64_t mi,
+                                                        int64_t j0, int64_t nj) {
   static_assert(kArgChunkLen == 64, "four lanes x four float4");
+  if (!STRIPS) {
+    i0 = j0 = 0;
+    lds = lde;
+    nj = mi;
+  }
   const int lane = threadIdx.x & 31, l = lane & 3;
   const float big = __int_as_float(0x7f800000);
   for (int r = threadIdx.x >> 5; r < kPickRows; r += 8) {
     const int64_t i = (int64_t)blockIdx.y * kPickRows + r;
-    if (i >= n) break;
+    if (i >= mi) break;
     const float *dr = De + i * lde;
 #pragma unroll 2
     for (int u = 0; u < 8; ++u) {
       const int64_t j = (int64_t)blockIdx.x * 64 + 8 * u + (lane >> 2);
-      const int c = j < n ? chunk[i * lde + j] : -1;
+      const int c = j < nj ? chunk[i * lds + j] : -1;
       const int k0 = c * kArgChunkLen + 4 * l;
       const float *wr = Wt + j * lde;
       float v[4][4];
@@ -380,25 +413,34 @@ __global__ void __launch_bounds__(256) pred_pick_kernel(const float *De, const f
         for (int q = 3; q >= 0; --q) k = v[t][q] == m ? k0 + 16 * t + q : k;
       k = min(k, __shfl_xor_sync(0xffffffffu, k, 1));
       k = min(k, __shfl_xor_sync(0xffffffffu, k, 2));
-      if (l == 0 && j < n) pred[i * ldp + j] = c >= 0 && i != j && m < big ? k : -1;
+      if (l == 0 && j < nj) pred[(i0 + i) * ldp + j0 + j] = c >= 0 && i0 + i != j0 + j && m < big ? k : -1;
     }
   }
 }
 
 int launch_chunked_f32(const void *d, int64_t ldd, const void *w, int64_t ldw, int *pred, int64_t ldp, int64_t n, float inf,
                        void *scratch, cudaStream_t s) {
-  const int64_t lde = enc_ld(n);
-  float *De = reinterpret_cast<float *>(scratch), *We = De + enc_bytes(n) / 4, *Wt = We + enc_bytes(n) / 4;
-  int *chunk = reinterpret_cast<int *>(Wt + enc_bytes(n) / 4);
-  const int64_t nt = cdiv(n, 32), cap = (int64_t)sm_count() * 8;
-  pred_clean_kernel<<<(unsigned)(nt * nt < cap ? nt * nt : cap), 256, 0, s>>>(
-      reinterpret_cast<const float *>(d), ldd, reinterpret_cast<const float *>(w), ldw, De, We, Wt, lde, n, inf,
-      status_word());
-  APSP_LAUNCH_CHECK();
-  int r;
-  if ((r = launch_arg_chunks(De, lde, We, lde, n, chunk, lde, s))) return r;
-  pred_pick_kernel<<<dim3((unsigned)cdiv(n, 64), (unsigned)cdiv(n, kPickRows)), 256, 0, s>>>(De, Wt, chunk, lde, pred, ldp, n);
-  APSP_LAUNCH_CHECK();
+  const int64_t edge = strip_edge(n), lde = enc_ld(n), lds = enc_ld(edge), cap = (int64_t)sm_count() * 8;
+  float *De = reinterpret_cast<float *>(scratch), *Wt = De + strip_bytes(edge, n) / 4, *We = Wt + strip_bytes(edge, n) / 4;
+  int *chunk = reinterpret_cast<int *>(We + strip_bytes(n, edge) / 4);
+  auto clean = edge < n ? pred_clean_kernel<true> : pred_clean_kernel<false>;
+  auto pick = edge < n ? pred_pick_kernel<true> : pred_pick_kernel<false>;
+  for (int64_t j0 = 0; j0 < n; j0 += edge) {
+    const int64_t nj = std::min(edge, n - j0);
+    for (int64_t i0 = 0; i0 < n; i0 += edge) {
+      const int64_t mi = std::min(edge, n - i0), wj = i0 == 0 ? nj : 0;
+      const int64_t tiles = cdiv(n, 32) * cdiv(wj ? n : mi, 32);
+      clean<<<(unsigned)std::min(tiles, cap), 256, 0, s>>>(reinterpret_cast<const float *>(d), ldd,
+                                                           reinterpret_cast<const float *>(w), ldw, De, We, Wt, lde, lds, n,
+                                                           i0, mi, j0, wj, inf, status_word());
+      APSP_LAUNCH_CHECK();
+      int r;
+      if ((r = launch_arg_chunks(De, lde, We, lds, mi, nj, n, chunk, lds, s))) return r;
+      pick<<<dim3((unsigned)cdiv(nj, 64), (unsigned)cdiv(mi, kPickRows)), 256, 0, s>>>(De, Wt, chunk, lde, lds, pred, ldp, i0,
+                                                                                       mi, j0, nj);
+      APSP_LAUNCH_CHECK();
+    }
+  }
   return APSP_OK;
 }
 
@@ -409,7 +451,7 @@ int launch_chunked_f32(const void *d, int64_t ldd, const void *w, int64_t ldw, i
 extern "C" size_t apsp_predecessors_workspace_bytes(int64_t n, int dtype) {
   using namespace apsp;
   if (n <= 0) return kFlagBytes;
-  if (dtype != APSP_I32) return kFlagBytes + (n >= kChunkedMinN ? chunked_bytes(n) : 0);
+  if (dtype != APSP_I32) return kFlagBytes + (n >= kChunkedMinN && n <= kChunkedMaxN ? chunked_bytes(n, strip_edge(n)) : 0);
   return kFlagBytes + 2 * enc_bytes(n);
 }
 
