@@ -241,12 +241,18 @@ class CostModel:
     def load(cls, path: str, device=None) -> "CostModel":
         with open(path) as f:
             d = json.load(f)
-        if d.get("in_dim") != IN_DIM or d.get("hidden") != HIDDEN:
+        params = d["params"]
+        if d.get("in_dim") == IN_DIM - 1 and d.get("hidden") == HIDDEN:
+            # A file from before the last feature (squaring's tile rounds): it gets weights of zero, which
+            # leave every prediction as it was.
+            at = (IN_DIM - 1) * HIDDEN
+            params = params[:at] + [0.0] * HIDDEN + params[at:]
+        elif d.get("in_dim") != IN_DIM or d.get("hidden") != HIDDEN:
             raise ValueError(f"{path}: a network of {d.get('in_dim')} features x {d.get('hidden')} units, "
                              f"not {IN_DIM} x {HIDDEN}; retrain it with planner.main()")
         m = cls(device=device)
         m.y_shift = d["y_shift"]
-        m.params = torch.tensor(d["params"], dtype=torch.float32, device=m.device)
+        m.params = torch.tensor(params, dtype=torch.float32, device=m.device)
         return m
 
 
