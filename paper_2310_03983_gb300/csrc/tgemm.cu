@@ -795,11 +795,13 @@ __global__ void __launch_bounds__(256) tgemm_generic_kernel(T *C, const T *A, co
     }
 }
 
+constexpr int64_t kGenericMaxM = 64 * 65535;  // 64 rows per block, in the grid's second dimension
+
 int launch_tgemm_generic(void *C, const void *A, const void *B, int64_t M, int64_t N, int64_t K, int64_t lda,
                          int64_t ldb, int64_t ldc, int dtype, bool acc, int inf_i, float inf_f, cudaStream_t s) {
   if (M == 0 || N == 0) return APSP_OK;
+  if (M > kGenericMaxM) return APSP_ERR_ARG;
   dim3 grid((unsigned)cdiv(N, 64), (unsigned)cdiv(M, 64));
-  if (grid.y > 65535) return APSP_ERR_ARG;
   if (dtype == APSP_I32)
     tgemm_generic_kernel<int><<<grid, 256, 0, s>>>((int *)C, (const int *)A, (const int *)B, M, N, K, lda, ldb, ldc,
                                                    acc, inf_i);
@@ -926,7 +928,9 @@ extern "C" int tropical_gemm(void *C, const void *A, const void *B, int64_t M, i
                        ldc % 4 == 0 && (K == 0 || (lda % 4 == 0 && ldb % 4 == 0));
   if (!aligned) {
     // Work on 16-byte aligned copies when the product is worth the passes and scratch may be taken
-    // here (no caller workspace, no capture); else the plain-load kernel.
+    // here (no caller workspace, no capture); else the plain-load kernel.  What that kernel refuses (M
+    // above kGenericMaxM) stays refused either way: whether a call is valid must not hang on free scratch.
+    if (M > kGenericMaxM) return APSP_ERR_ARG;
     const int64_t least = dtype == APSP_F32 ? kRepackMinPairsF32 : kRepackMinPairsI32;
     if (!ws && K > 0 && M * N > least / K) {
       const int done = tropical_gemm_repacked(C, A, B, M, N, K, lda, ldb, ldc, dtype, inf, accumulate, s);
