@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(kFThreads, 1) gemm64_kernel(const __grid_const
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kProducerRegs));
     if (lane != 0 || g >= a.groups) return;
     if ((threadIdx.x >> 5) % 4 < 2) {  // ------------------------- loads -------------------------
-      const int chunks = (a.K + kFB - 1) / kFB, step = gridDim.x * a.groups;
+      const int chunks = (a.K - 1) / kFB + 1, step = gridDim.x * a.groups;  // K may be INT32_MAX
       uint32_t issued = 0, pars = 0, c = 0;  // c: chunks issued so far
       int m = 0, seen = 0;                   // items so far; stages known to have changed something
       bool ok = true;
