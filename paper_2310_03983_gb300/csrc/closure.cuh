@@ -1,9 +1,14 @@
 // closure.cuh -- internal interfaces between the closure drivers (fw.cu, rkleene.cu).
 #pragma once
 
+#include "fine.cuh"
 #include "tgemm.cuh"
 
 namespace apsp {
+
+// The counters' place in the block of bound words at the front of a closure's workspace.
+constexpr int kCounterWord = 40, kCounterWords = kFineWords > 3 ? kFineWords : 3;
+static_assert((kCounterWord + kCounterWords) * sizeof(int) <= kFlagBytes, "bound words");
 
 // Device bound words of a closure (see TileProblem::wmax): w[0] = largest finite weight,
 // mult = n - 1 of the whole graph.  w == nullptr for float32.  cert (may be null: then w[0])
@@ -14,8 +19,9 @@ struct Bound {
   const int *w;
   int64_t mult;
   const int *cert = nullptr;
-  // Three device words, zero at the start: the counters of phase 3's dynamic scheduling
-  // (TileProblem::tile_counter; null: static order, and phases 1 and 2 in launches of their own).
+  // kCounterWords device words, zero at the start and between launches: the counters of phase 3's dynamic
+  // scheduling (TileProblem::tile_counter, three words) or of the 64-vertex-block closure (fine.cu).
+  // Null: static order, and phases 1 and 2 in launches of their own.
   int *counters = nullptr;
 };
 

@@ -482,7 +482,7 @@ int closure_entry(int algo, void *d, int64_t n, int64_t ld, int dtype, const voi
   wsp += kFlagBytes;
   if (cudaMemsetAsync(words, 0, kFlagBytes, s) != cudaSuccess) r = APSP_ERR_CUDA;
   Bound bound = {dtype == APSP_I32 ? words : nullptr, n - 1};
-  bound.counters = words + 40;  // three words, zeroed with the rest of the block
+  bound.counters = words + kCounterWord;  // zeroed with the rest of the block
   void *work = d;
   int64_t ldw = ld;
   if (ld % 4 != 0) {  // repack into an aligned copy at the front of the workspace
