@@ -46,7 +46,6 @@ struct FineArgs {
   int inf;        // bits of the "no edge" value
   const int *wmax;
   int64_t wmult;
-  const int *run_if;
   int *counters;
   unsigned int *status;
 };
@@ -75,7 +74,7 @@ struct StageCounts {
 };
 __device__ __forceinline__ StageCounts stage_counts(int nt, int s) {
   StageCounts c = {0, 0, 0, 0};
-  if (s > nt || (s == nt && nt == 1)) return c;
+  if (s > nt) return c;
   c.close = s < nt;
   c.dep = s > 0 && s < nt ? 2 * nt - 4 : 0;
   c.rest = s == 0 ? 0 : s < nt ? (nt - 2) * (nt - 2) : (nt - 1) * (nt - 1);
@@ -301,7 +300,6 @@ __global__ void __launch_bounds__(kFThreads, 1)
   __syncthreads();
   pdl_wait();  // after the set-up, before any global memory access
   pdl_trigger();
-  if (a.run_if && !*a.run_if) return;
 
   if (wg == kFGroups) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kProducerRegs));
@@ -504,7 +502,7 @@ static int fine_maps(CUtensorMap *mA, CUtensorMap *mB, const void *d, int64_t ro
 }
 
 int fine_closure(void *d, int64_t n, int64_t ld, int dtype, int inf_i, const int *wmax, int64_t wmult,
-                 const int *run_if, int *counters, int trace_class, cudaStream_t s) {
+                 int *counters, int trace_class, cudaStream_t s) {
   CUtensorMap mA, mB;
   int r;
   if ((r = fine_maps(&mA, &mB, d, n, n, ld, dtype))) return r;
@@ -517,14 +515,12 @@ int fine_closure(void *d, int64_t n, int64_t ld, int dtype, int inf_i, const int
   a.inf = dtype == APSP_F32 ? 0x7f800000 : inf_i;
   a.wmax = dtype == APSP_F32 ? nullptr : wmax;
   a.wmult = wmult;
-  a.run_if = run_if;
   a.counters = counters;
   a.status = status_word();
   a.groups = fine_groups((int64_t)(a.nt - 1) * (a.nt - 1), sm_count());
   a.rest1 = 2 * a.nt - 3;
-  // nt + 1 stages over as many launches as the 128-vertex loop makes (1, or 2 + one per block).
-  const int64_t nb = cdiv(n, kBM);
-  const int stages = a.nt == 1 ? 1 : a.nt + 1, launches = nb == 1 ? 1 : (int)nb + 2;
+  // nt + 1 stages over as many launches as the 128-vertex loop makes: two, and one per 128 vertices.
+  const int stages = a.nt + 1, launches = (int)cdiv(n, kBM) + 2;
   for (int l = 0; l < launches; ++l) {
     a.s0 = (int)((int64_t)stages * l / launches);
     a.s1 = (int)((int64_t)stages * (l + 1) / launches);

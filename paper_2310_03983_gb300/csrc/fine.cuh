@@ -16,12 +16,11 @@ constexpr int64_t kFineMinN = 128, kFineMaxN = 3200;
 constexpr int kFineMaxStages = 8;  // of one launch
 constexpr int kFineWords = 2 + 2 * kFineMaxStages;
 
-// Closes the n x n block at d (16-byte aligned, ld % 4 == 0, normalised) in place with
-// 1 + (number of 128-vertex blocks) launches after the first (one launch when n <= 128), the
-// launch structure of the 128-vertex loop.  wmax / wmult: the bound of the exact fp32 sequence for int32 storage (null: float32).
-// run_if (may be null): every launch returns at once unless *run_if is set.
+// Closes the n x n block at d (16-byte aligned, ld % 4 == 0, normalised, n > kFineMinN) in place in two
+// launches and one per 128 vertices, as the 128-vertex loop does.  wmax / wmult: the bound of the exact
+// fp32 sequence for int32 storage (null: float32).
 int fine_closure(void *d, int64_t n, int64_t ld, int dtype, int inf_i, const int *wmax, int64_t wmult,
-                 const int *run_if, int *counters, int trace_class, cudaStream_t s);
+                 int *counters, int trace_class, cudaStream_t s);
 
 // The same for many graphs in lockstep, staged one below the other in d (rows x ld, each graph padded to
 // whole 128-vertex blocks with isolated vertices, groups by decreasing nb; gsize: device, vertices of

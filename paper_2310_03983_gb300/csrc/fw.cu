@@ -231,8 +231,8 @@ static int fw_loop(void *d, int64_t n, int64_t ld, int dtype, const CUtensorMap 
                    int *counters = nullptr) {
   int r;
   const int64_t nb = p.nb;
-  if (counters && n <= kFineMaxN && n > kFineMinN)
-    return fine_closure(d, n, ld, dtype, p.inf_i, p.wmax, p.wmult, run_if, counters, trace_class, s);
+  if (counters && !run_if && n <= kFineMaxN && n > kFineMinN)
+    return fine_closure(d, n, ld, dtype, p.inf_i, p.wmax, p.wmult, counters, trace_class, s);
   p.run_if = run_if;
   p.trace_class = trace_class;
   for (int64_t kb = 0; kb < nb; ++kb) {
