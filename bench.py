@@ -88,7 +88,16 @@ MAX_SM_MHZ = 2070.0
 # they were taken on (hash below).
 PHASE3_DRAM_BYTES_PER_C_ELEM = {1: 7.605, 2: 7.833}
 PHASE3_TRAFFIC_SRC_HASH = "08cad5469c393595"
-TGEMM_SOURCES = ("tgemm.cu", "tgemm.cuh", "slab.cuh", "common.cuh")
+TGEMM_SOURCES = ("tgemm.cu", "tgemm.cuh", "slab.cuh", "diag.cuh", "common.cuh")
+
+
+def dominant_kernel(w, n, mode):
+    """The kernel whose traced launches the roofline line adds up."""
+    if mode == 0:
+        return "tgemm_kernel and gemm64_kernel (products)" if w["algo"] == "rkleene" else "tgemm_kernel (product)"
+    if w["algo"] == "fw" and 128 < n <= 3200:
+        return "fine_fw_kernel (64-vertex blocks: diagonal closures, panels and remaining tiles)"
+    return "tgemm_kernel (FW phase 3)"
 
 
 def tgemm_src_hash():
@@ -614,7 +623,7 @@ def run_ours(args, w, rank, world, local_rank):
         "dtype": dtype_tag,
         "arith": arith,
         "data": "synthetic", "config": config_of(args, w, world),
-        "roofline": {"bound": "alu", "kernel": {0: "tgemm_kernel (product)", 2: "tgemm_kernel (FW phase 3)"}[dom_mode],
+        "roofline": {"bound": "alu", "kernel": dominant_kernel(w, n, dom_mode),
                      "achieved": round(achieved, 2) if achieved else None, "peak": round(peak_max, 2),
                      "unit": "Tops/s", "frac": round(achieved / peak_max, 4) if achieved else None,
                      "frac_at_observed_clock": (round(achieved / (peak_max * sm_mhz / MAX_SM_MHZ), 4)

@@ -26,10 +26,11 @@ __device__ __forceinline__ void flag_status(unsigned int *st, int code) {
   if (st) atomicOr(st, 1u << code);
 }
 
-// Iteration limit of every spin-wait on an mbarrier.  The longest legitimate wait in these
-// kernels is one tile of work (tens of microseconds); 2^24 try_wait calls take between a
-// fraction of a second and a few seconds, so a wait that cannot complete ends the kernel
-// with APSP_ERR_TIMEOUT instead of hanging the GPU.
+// Iteration limit of every spin-wait, on an mbarrier or a device counter.  The longest legitimate
+// wait is one tile of work in most kernels (tens of microseconds) and, in the kernels that run several
+// dependent steps (fine.cu, gemm64.cu), one whole step: a product of repeated squaring takes up to
+// two milliseconds (n = 2896).  2^24 polls take between a fraction of a second and a few seconds, so
+// a wait that cannot complete ends the kernel with APSP_ERR_TIMEOUT instead of hanging the GPU.
 constexpr uint32_t kSpinLimit = 1u << 24;
 
 // Cap of the packed 16-bit (min,+) arithmetic: values at or above it mean "at least the cap";

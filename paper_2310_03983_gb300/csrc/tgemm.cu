@@ -677,8 +677,8 @@ __device__ __forceinline__ bool fits16(const int *words) {
   return (int64_t)words[0] + (int64_t)words[1] < kCap16;
 }
 __device__ __forceinline__ int cap16(int v, int inf) { return v >= inf ? kCap16 : v; }
-// The operands' rows are 16-byte aligned (the engine's own condition).
 
+// The packing kernels' operands have 16-byte aligned rows (the engine's own condition).
 __global__ void __launch_bounds__(256) pack16_a_kernel(const int *A, int64_t lda, int64_t M, int64_t K, int *A16,
                                                        int64_t ld16, int inf, int *words) {
   pdl_wait();
