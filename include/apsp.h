@@ -239,8 +239,10 @@ int apsp_rkleene_noalloc(void *d, int64_t n, int64_t ld, int dtype, const void *
  * offsets, ns, lds and order are DEVICE arrays of `count` entries; ns_host (optional, host) is
  * a copy of ns that lets the library pick the launch shape: when some graph would take longer
  * alone than the average work per SM, the kernel runs as thread-block clusters that close
- * such graphs together; otherwise one CTA per graph on every SM (NULL: clusters).  pool must be 16-byte
- * aligned; every lds[g] and offsets[g] must be a multiple of 4 and lds[g] >= ns[g]: a graph
+ * such graphs together, and the other graphs above 128 vertices too when the batch ends sooner that
+ * way; otherwise one CTA per graph on every SM (NULL: clusters).  An int32 graph whose (n - 1) *
+ * largest finite weight is below 2^24 is closed in exact fp32 arithmetic on its bit patterns, diagonal
+ * tiles included, others in int32.  pool must be 16-byte aligned; every lds[g] and offsets[g] must be a multiple of 4 and lds[g] >= ns[g]: a graph
  * that breaks this, or an order entry outside [0, count), is skipped and sets APSP_ERR_ARG
  * in the device status word (the rest of the batch is still closed).  ns[g] <= 0 is skipped.
  * The workspace holds the work-queue counter (apsp_batched_workspace_bytes); with the room
@@ -259,7 +261,7 @@ size_t apsp_batched_workspace_bytes(int64_t count);
  * whose certificate fails).  When a step of all staged graphs together is at most 12 tiles of 64 x 64
  * per SM, they are closed in 32 bits over 64-vertex blocks instead.  Every other graph goes to the
  * persistent kernel.  Returns
- * apsp_batched_workspace_bytes(count) when no graph qualifies or dtype is APSP_F32.  The
+ * apsp_batched_workspace_bytes(count) when no graph qualifies.  The
  * staged path runs only when apsp_batched gets ns_host, a caller workspace of at least this
  * size and a sentinel above 0x3FFF; a staged graph whose device size, leading dimension or
  * offset disagree with ns_host or the layout rules is left untouched and sets APSP_ERR_ARG. */

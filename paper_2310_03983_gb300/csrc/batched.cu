@@ -439,8 +439,8 @@ __global__ void __launch_bounds__(kBThreads, 1) batched_kernel(const BatchArgs a
     // way.  Left alone, the largest of them takes lone_cost on one CTA while the other CTAs close the
     // graphs of one tile; on clusters, every CTA has its share of both (the last of which ends half
     // a graph late on average).  Measured (int32, us, on clusters / alone; share of the line below): 16 graphs of
-    // 256 beside 400 of 64 190 / 235 (0.69), 19 beside 1000 of 32 207 / 237 (0.90), 16 of 200 beside 400 of 128
-    // 229 / 196 (1.23), 19 of 256 beside 1000 of 100 363 / 288 (1.76).
+    // 256 beside 400 of 64 190 / 235 (0.70), 19 beside 1000 of 32 207 / 237 (0.90), 16 of 200 beside 400 of 128
+    // 229 / 196 (1.24), 19 of 256 beside 1000 of 100 363 / 288 (1.72).
     // Every CTA adds in the same order, so all come to the same choice.
     const int ntile = s_ntile;
     if (ntile > nbig && ntile <= min((int)gridDim.x / csize, kBThreads)) {
